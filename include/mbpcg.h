@@ -58,7 +58,10 @@ typedef enum { MBPCG_PRECOND_NONE = 0, MBPCG_PRECOND_JACOBI = 1 } mbpcg_precond;
  * paper's baseline, Section 4), s ignored. */
 typedef enum { MBPCG_ALGO_MBPCG = 0, MBPCG_ALGO_CG = 1 } mbpcg_algo;
 
-/* Arithmetic of the n-proportional work. FP64: everything in double precision on the FP64 pipe.
+/* Arithmetic of the n-proportional work. FP64: everything in double precision, on the FP64 pipe; in CSR
+ * MBPCG solves with at least 2^17 values per padded block (n times the padded width, width >= 4) the block
+ * update, and for wider blocks the W/P update and the Gram matrices, form their s x s contractions by
+ * exact digit splitting on the tensor cores, with the accuracy of an FP64 sum (csrc/rows_mma.cuh).
  * MIXED_FP32 (MBPCG only; CSR or dense A): the inner solves keep the n x s blocks and the (scaled)
  * matrix in FP32 (a dense A adds an FP32 copy, n x round_up(n, 32) floats, to the workspace) and do
  * the products and block updates in FP32 with FP32 accumulation; the s x s

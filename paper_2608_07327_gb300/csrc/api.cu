@@ -58,6 +58,9 @@ struct Dims {
   int mixed;  // MBPCG_MIXED_FP32: FP32 blocks and values in the inner solve
   int cg_fused;  // dense CG in one launch per iteration (k_cg_dense_iter)
   int nb_cg;     // its CTAs (a multiple of the cluster size)
+  int mx;        // the block update on the tensor cores (rows_mma.cuh), with nb_mx CTAs
+  int mx_pw, mx_gram;  // and the W/P update, the Gram of the product
+  int nb_mx;
 };
 
 int num_sms() {
@@ -95,7 +98,28 @@ Dims make_dims(int n, long long nnz, int s, int algo, int dense, int sms) {
   d.cg_fused = (dense && algo == MBPCG_ALGO_CG && cg_dense_fused_ok(n)) ? 1 : 0;
   d.nb_cg = d.cg_fused ? cg_dense_grid(n, sm) : 0;
   if (d.nb_cg > d.nbmax) d.nbmax = d.nb_cg;
+  d.mx = d.mx_pw = d.mx_gram = d.nb_mx = 0;
   return d;
+}
+
+// The tensor-core row passes (rows_mma.cuh) of a CSR MBPCG handle in FP64, two persistent CTAs per SM,
+// which take 8 tiles of 16 view rows at a time. Dense handles keep the FP64 passes: their time is the
+// product's, and their iteration counts, past the exact-termination bound, move with every rounding.
+// The lines are where the two sides measured alike (us per iteration of what each replaces):
+//   kp * n >= 2^17: Poisson 64^2, kp = 4 (2^14): 17.8 against 7.4 for the block update; diffusion 24^3, kp =
+//     16 (2^17.8): 20 against 28; diffusion 41^3, kp = 4 (2^18): 19 against 26;
+//   W/P update from kp = 8 (table in rows_mma.cuh: 92 against 77 at kp = 4, 88 against 129 at 8);
+//   Gram of the product from kp = 16 and kp * n >= 2^19 (kp = 8: 201 with the product against 182 fused;
+//     diffusion 24^3, kp = 32 (2^18.8): 22 against 24; kp = 16 (2^17.8): 15 against 10.6).
+void apply_mx(Dims& d) {
+  const long long values = (long long)d.n * d.kp;
+  if (d.dense || d.algo != MBPCG_ALGO_MBPCG || d.kp < 4 || values < (1LL << 17)) return;
+  d.mx = 1;
+  d.mx_pw = d.kp >= 8;
+  d.mx_gram = d.kp >= 16 && values >= (1LL << 19);
+  const long long view = (values + 15) / 16, want = (view + 127) / 128;
+  d.nb_mx = (int)(want < 2LL * d.sms ? want : 2LL * d.sms);
+  if (d.nb_mx > d.nbmax) d.nbmax = d.nb_mx;
 }
 
 // Partial-sum slots of a solver handle also hold the weighted Gram V^T D^2 V of the
@@ -635,14 +659,18 @@ void enqueue_product(mbpcg_ctx* h, const RowOps* ops, const double* X, double* Y
     ops->dense(h->stream, dm.nb_dense, dm.n, h->A, X, Y, st, &h->st->kerr);
     if (gram) ops->gram(h->stream, dm.nb, dm.n, X, Y, h->part, dm.pstride, st);
   } else if (h->prod64 == MBPCG_PRODUCT_CSR_TILED) {
-    spmm_tiled(h->stream, dm.kp, dm.nb, dm.n, h->rp, h->av, h->plan, X, Y, h->part, dm.pstride, st, gram);
+    spmm_tiled(h->stream, dm.kp, dm.nb, dm.n, h->rp, h->av, h->plan, X, Y, h->part, dm.pstride, st,
+               gram && !dm.mx_gram);
+    if (gram && dm.mx_gram) ops->gram_mx(h->stream, dm.nb_mx, dm.n, X, Y, nullptr, h->part, dm.pstride, st);
   } else {
-    ops->spmm(h->stream, dm.nb, dm.n, h->rp, h->ci, h->av, X, Y, h->part, dm.pstride, st, gram);
+    ops->spmm(h->stream, dm.nb, dm.n, h->rp, h->ci, h->av, X, Y, h->part, dm.pstride, st, gram && !dm.mx_gram);
+    if (gram && dm.mx_gram) ops->gram_mx(h->stream, dm.nb_mx, dm.n, X, Y, nullptr, h->part, dm.pstride, st);
   }
 }
 
-void enqueue_reduce(mbpcg_ctx* h, int nent, const SolveState* st) {
-  launch_reduce(h->stream, h->part, h->dm.nb, h->dm.pstride, h->red, nent, st);
+// red[e0 .. e0 + nent) from the partials of the FP64 row kernels, or of the tensor-core ones (mx).
+void enqueue_reduce(mbpcg_ctx* h, int nent, const SolveState* st, int mx = 0, int e0 = 0) {
+  launch_reduce(h->stream, h->part + e0, mx ? h->dm.nb_mx : h->dm.nb, h->dm.pstride, h->red + e0, nent, st);
 }
 
 void enqueue_true_residual(mbpcg_ctx* h) {
@@ -665,10 +693,12 @@ void enqueue_mbpcg_setup(mbpcg_ctx* h) {
   ops->setup_norms(h->stream, dm.nb, n, h->rhs, h->d, h->bs, h->Q, h->part, dm.pstride);
   enqueue_reduce(h, 3, nullptr);
   k_small_setup<<<1, 1, 0, h->stream>>>(h->st, h->red);
-  ops->init(h->stream, dm.nb, n, h->s, h->U, h->Q, h->bs, h->X0, h->Xt, h->R, h->part, dm.pstride, h->st);
-  enqueue_reduce(h, npack(kp), nullptr);
+  ops->init(h->stream, dm.nb, n, h->s, h->U, h->Q, h->bs, h->X0, h->Xt, h->R, h->part, dm.pstride, h->st, !dm.mx);
+  if (dm.mx) ops->gram_mx(h->stream, dm.nb_mx, n, h->R, h->R, nullptr, h->part, dm.pstride, nullptr);
+  enqueue_reduce(h, npack(kp), nullptr, dm.mx);
   launch_small_sigma(h->stream, kp, h->st, h->red, h->Sigma, h->SigmaInv);
-  ops->pw(h->stream, dm.nb, n, h->R, h->W, h->P, h->SigmaInv, nullptr, nullptr, 1, dm.tc ? h->oz_ep : nullptr);
+  if (dm.mx_pw) ops->pw_mx(h->stream, dm.nb_mx, n, h->R, h->W, h->P, h->SigmaInv, nullptr, nullptr, 1);
+  else ops->pw(h->stream, dm.nb, n, h->R, h->W, h->P, h->SigmaInv, nullptr, nullptr, 1, dm.tc ? h->oz_ep : nullptr);
 }
 
 void enqueue_mbpcg_body(mbpcg_ctx* h) {
@@ -679,28 +709,36 @@ void enqueue_mbpcg_body(mbpcg_ctx* h) {
   const bool tcrows = h->rp3 != nullptr && !h->rfree;
   double *Y0 = h->rp3, *Y1 = Y0 + (size_t)n * kp, *Y2 = Y1 + (size_t)n * kp;
   enqueue_product(h, ops, h->P, h->Q, 1, h->st);
-  enqueue_reduce(h, npack(kp), h->st);
+  enqueue_reduce(h, npack(kp), h->st, dm.mx_gram);
   launch_small_xi(h->stream, kp, h->st, h->red, h->Sigma, h->Xi, h->T);
   if (tcrows) {
     const RowProdJobs jb = {{{h->P, h->T, 0, Y0}, {h->Q, h->T, 0, Y1}, {h->Q, h->Xi, 0, Y2}}};
     rowprod_tc(h->stream, n, kp, jb, 3, h->st, 0, &h->st->kerr);
     ops->axpy_pre(h->stream, dm.nb, n, Y0, Y1, Y2, h->W, h->R, h->Xt, h->V, h->wdiag, h->part, dm.pstride, h->st);
+  } else if (dm.mx) {
+    ops->axpy_mx(h->stream, dm.nb_mx, n, h->P, h->Q, h->W, h->R, h->Xt, h->V, h->T, h->Xi, h->wdiag, h->part,
+                 dm.pstride, h->st, h->rfree);
+    ops->gram_mx(h->stream, dm.nb_mx, n, h->V, h->V, nullptr, h->part, dm.pstride, h->st);
+    if (h->rfree && h->wdiag != nullptr)  // V^T D^2 V
+      ops->gram_mx(h->stream, dm.nb_mx, n, h->V, h->V, h->wdiag, h->part + npack(kp) + kp, dm.pstride, h->st);
   } else {
     ops->axpy(h->stream, dm.nb, n, h->P, h->Q, h->W, h->R, h->Xt, h->V, h->T, h->Xi, h->wdiag, h->part, dm.pstride,
               h->st, h->rfree);
   }
   if (h->rfree) {  // nu_j from the Gram of V (weighted with scaling) and Sigma
     const bool w = h->wdiag != nullptr;
-    enqueue_reduce(h, w ? 2 * npack(kp) + kp : npack(kp), h->st);
+    enqueue_reduce(h, w ? 2 * npack(kp) + kp : npack(kp), h->st, dm.mx);
     k_small_nu<<<kp, 32, 0, h->stream>>>(h->st, h->red, h->Sigma, kp, w ? npack(kp) + kp : 0);
   } else {
-    enqueue_reduce(h, npack(kp) + kp, h->st);
+    enqueue_reduce(h, npack(kp) + kp, h->st, dm.mx);
   }
   launch_small_zeta(h->stream, kp, h->st, h->red, h->Sigma, h->Zeta, h->ZetaInv, h->cond, h->use_cond);
   if (tcrows) {
     const RowProdJobs jb = {{{h->V, h->ZetaInv, 0, Y0}, {h->P, h->Zeta, 1, Y1}, {nullptr, nullptr, 0, nullptr}}};
     rowprod_tc(h->stream, n, kp, jb, 2, h->st, 1, &h->st->kerr);
     ops->pw_pre(h->stream, n, Y0, Y1, h->W, h->P, h->st, h->oz_ep);
+  } else if (dm.mx_pw) {
+    ops->pw_mx(h->stream, dm.nb_mx, n, h->V, h->W, h->P, h->ZetaInv, h->Zeta, h->st, 0);
   } else {
     ops->pw(h->stream, dm.nb, n, h->V, h->W, h->P, h->ZetaInv, h->Zeta, h->st, 0, dm.tc ? h->oz_ep : nullptr);
   }
@@ -711,8 +749,14 @@ void enqueue_mbpcg_exit(mbpcg_ctx* h) {
   const RowOps* ops = row_ops(dm.kp);
   const int kp = dm.kp, n = dm.n;
   if (h->rfree) ops->rsig(h->stream, dm.nb, n, h->V, h->W, h->Sigma, h->R, h->st);
-  ops->ls_gram(h->stream, dm.nb, n, h->R, h->rhs, h->sqd, h->part, dm.pstride);
-  enqueue_reduce(h, npack(kp) + kp + 1, nullptr);
+  ops->ls_gram(h->stream, dm.nb, n, h->R, h->rhs, h->sqd, h->part, dm.pstride, !dm.mx);
+  if (dm.mx) {  // (D R)^T (D R) = R^T D^2 R; the other entries from their own partials
+    ops->gram_mx(h->stream, dm.nb_mx, n, h->R, h->R, h->wdiag, h->part, dm.pstride, nullptr);
+    enqueue_reduce(h, npack(kp), nullptr, 1);
+    enqueue_reduce(h, kp + 1, nullptr, 0, npack(kp));
+  } else {
+    enqueue_reduce(h, npack(kp) + kp + 1, nullptr);
+  }
   k_small_ls<<<1, kSmallThreads, 0, h->stream>>>(h->st, h->red, kp, h->c);
   ops->combine(h->stream, dm.nb, n, h->s, h->Xt, h->X0, h->c, h->d, h->x);
   enqueue_true_residual(h);
@@ -1084,6 +1128,7 @@ size_t mbpcg_workspace_size_csr(int32_t n, int64_t nnz, int32_t s, int32_t algo,
   if (n < 1 || nnz < 0) return 0;
   Dims dm = make_dims(n, nnz, s, algo, 0, num_sms());
   if (precision == MBPCG_MIXED_FP32 && algo == MBPCG_ALGO_MBPCG) apply_mixed(dm);
+  else apply_mx(dm);
   widen_for_handle(dm);
   return make_layout(dm).total;
 }
@@ -1112,6 +1157,7 @@ int mbpcg_create_csr(mbpcg_handle* out, int32_t n, int64_t nnz, const int32_t* r
   mbpcg_ctx* h = nullptr;
   Dims dm = make_dims(n, nnz, s, algo, 0, sms);
   if (precision == MBPCG_MIXED_FP32) apply_mixed(dm);
+  else apply_mx(dm);
   widen_for_handle(dm);
   rc = alloc_handle(&h, dm, s, precond, algo, precision, seed, workspace, workspace_bytes, stream);
   if (rc) {

@@ -41,9 +41,9 @@ struct RowOps {
   void (*setup_norms)(cudaStream_t, int nb, int n, const double* rhs, const double* d, double* bs,
                       const double* AU, double* part, int pstride);
   void (*init)(cudaStream_t, int nb, int n, int s, const double* U, const double* AU, const double* bs, double* X0,
-               double* Xt, double* R, double* part, int pstride, const SolveState* st);
+               double* Xt, double* R, double* part, int pstride, const SolveState* st, int gram);
   void (*ls_gram)(cudaStream_t, int nb, int n, const double* R, const double* rhs, const double* sqd, double* part,
-                  int pstride);
+                  int pstride, int gram);
   void (*combine)(cudaStream_t, int nb, int n, int s, const double* Xt, const double* X0, const double* c,
                   const double* d, double* x);
   void (*gen_u)(cudaStream_t, int n, int s, unsigned long long seed, double* U);
@@ -56,6 +56,15 @@ struct RowOps {
                    const SolveState* st);
   void (*pw_pre)(cudaStream_t, int n, const double* VZi, const double* PZt, double* W, double* P, const SolveState* st,
                  int* emax);
+  // the row passes on the tensor cores (rows_mma.cuh; KP >= 4): the Gram X^T Y (X weighted by w row by
+  // row, or NULL), the block update without its Gram, the W/P update
+  void (*gram_mx)(cudaStream_t, int nb, int n, const double* X, const double* Y, const double* w, double* part,
+                  int pstride, const SolveState* st);
+  void (*axpy_mx)(cudaStream_t, int nb, int n, const double* P, const double* Q, const double* W, double* R,
+                  double* Xt, double* V, const double* T, const double* Xi, const double* wdiag, double* part,
+                  int pstride, const SolveState* st, int rfree);
+  void (*pw_mx)(cudaStream_t, int nb, int n, const double* V, double* W, double* P, const double* Zinv,
+                const double* Z, const SolveState* st, int setp);
 };
 
 const RowOps* row_ops_kp1();

@@ -666,22 +666,22 @@ k_setup_norms(int n, const double* __restrict__ rhs, const double* __restrict__ 
 }
 
 // X0 = scale U;  X~ = 0;  R = B~ = bs 1^T - scale (A U)  (columns < s; padded columns stay 0);
-// and the CTA partials of R^T R for the set-up Cholesky QR (W^0, Sigma^0 = qr(R^0)).
-template <int KP>
+// and, when GRAM, the CTA partials of R^T R for the set-up Cholesky QR (W^0, Sigma^0 = qr(R^0)).
+template <int KP, bool GRAM>
 __global__ void __launch_bounds__(kThreads)
 k_init(int n, int s, const double* __restrict__ U, const double* __restrict__ AU, const double* __restrict__ bs,
        double* __restrict__ X0, double* __restrict__ Xt, double* __restrict__ R, double* __restrict__ part,
        int pstride, const SolveState* __restrict__ st) {
   using C = Cfg<KP>;
   using G = GramTile<KP>;
-  __shared__ __align__(16) double Rs[C::ROWS * KP];
-  __shared__ __align__(16) double red[G::RED];
+  __shared__ __align__(16) double Rs[GRAM ? C::ROWS * KP : 2];
+  __shared__ __align__(16) double red[GRAM ? G::RED : 2];
   const double scale = st->scale;
   int r0, r1;
   row_range(n, r0, r1);
   const int tid = threadIdx.x, rl = tid / C::TPR, j0 = (tid % C::TPR) * C::CPT;
   G g;
-  g.init(tid);
+  if constexpr (GRAM) g.init(tid);
   for (int base = r0; base < r1; base += C::ROWS) {
     const int i = base + rl;
     double rv[C::CPT];
@@ -702,33 +702,36 @@ k_init(int n, int s, const double* __restrict__ U, const double* __restrict__ AU
       stv<C::CPT>(Xt + (size_t)i * KP + j0, z);
       stv<C::CPT>(R + (size_t)i * KP + j0, rv);
     }
+    if constexpr (GRAM) {
 #pragma unroll
-    for (int c = 0; c < C::CPT; ++c) Rs[rl * KP + j0 + c] = rv[c];
-    __syncthreads();
-    g.accumulate(Rs, Rs, min(C::ROWS, r1 - base));
-    __syncthreads();
+      for (int c = 0; c < C::CPT; ++c) Rs[rl * KP + j0 + c] = rv[c];
+      __syncthreads();
+      g.accumulate(Rs, Rs, min(C::ROWS, r1 - base));
+      __syncthreads();
+    }
   }
-  g.finish(red, part + (size_t)blockIdx.x * pstride);
+  if constexpr (GRAM) g.finish(red, part + (size_t)blockIdx.x * pstride);
 }
 
 // ------------------------------------------------------------------------------------------------
 // Exit (least-squares combination of Section 2): CTA partials of the Gram of M = [rhs | D R] in
 // the original metric: upper triangle of (DR)^T (DR) at [0, NPACK), rhs^T (DR)_j at NPACK + j,
-// rhs^T rhs at NPACK + KP. sqd = sqrt(diag A) (= D), or NULL without scaling.
-template <int KP>
+// rhs^T rhs at NPACK + KP. sqd = sqrt(diag A) (= D), or NULL without scaling. GRAM = false: without the
+// first.
+template <int KP, bool GRAM>
 __global__ void __launch_bounds__(kThreads)
 k_ls_gram(int n, const double* __restrict__ R, const double* __restrict__ rhs, const double* __restrict__ sqd,
           double* __restrict__ part, int pstride) {
   using C = Cfg<KP>;
   using G = GramTile<KP>;
   constexpr int RED = (G::RED > C::ROWS * (KP + 1)) ? G::RED : C::ROWS * (KP + 1);
-  __shared__ __align__(16) double Ms[C::ROWS * KP];
+  __shared__ __align__(16) double Ms[GRAM ? C::ROWS * KP : 2];
   __shared__ __align__(16) double red[RED];
   int r0, r1;
   row_range(n, r0, r1);
   const int tid = threadIdx.x, rl = tid / C::TPR, j0 = (tid % C::TPR) * C::CPT;
   G g;
-  g.init(tid);
+  if constexpr (GRAM) g.init(tid);
   double br[C::CPT], bb = 0.0;
 #pragma unroll
   for (int c = 0; c < C::CPT; ++c) br[c] = 0.0;
@@ -748,14 +751,16 @@ k_ls_gram(int n, const double* __restrict__ R, const double* __restrict__ rhs, c
       }
       if (j0 == 0) bb = fma(b, b, bb);
     }
+    if constexpr (GRAM) {
 #pragma unroll
-    for (int c = 0; c < C::CPT; ++c) Ms[rl * KP + j0 + c] = mv[c];
-    __syncthreads();
-    g.accumulate(Ms, Ms, min(C::ROWS, r1 - base));
-    __syncthreads();
+      for (int c = 0; c < C::CPT; ++c) Ms[rl * KP + j0 + c] = mv[c];
+      __syncthreads();
+      g.accumulate(Ms, Ms, min(C::ROWS, r1 - base));
+      __syncthreads();
+    }
   }
   double* out = part + (size_t)blockIdx.x * pstride;
-  g.finish(red, out);
+  if constexpr (GRAM) g.finish(red, out);
 #pragma unroll
   for (int c = 0; c < C::CPT; ++c) red[rl * (KP + 1) + j0 + c] = br[c];
   if (j0 == 0) red[rl * (KP + 1) + KP] = bb;

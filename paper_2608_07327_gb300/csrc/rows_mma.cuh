@@ -1,0 +1,609 @@
+// The row passes of the CSR handles (block update, W/P update, Gram matrices) on the FP16 tensor cores
+// with FP64 accuracy, by exact digit splitting (Ozaki et al., "Error-free transformations of matrix
+// multiplication by using fast routines of matrix multiplication and its applications", Numer.
+// Algorithms 2012), from registers to registers (mma.sync.m16n8k16).
+//
+// Why. GB300 issues 2 FP64 lanes per clock per SM: at 16 columns a row of the block update is 768 + 144
+// FP64 FMAs, and the FP64 pipe made these passes 10 times slower than their bytes. Here the contractions
+// are integer digit products on the tensor cores, the splitting and recombination are integer
+// operations, and the FP64 pipe keeps one add per output and the norms; the three pipes run side by
+// side. What binds now is the integer work: about 50 operations per value split or combined, half of them
+// on the 16-lane ALU (54 % busy). Measured (us per launch, FP64 pipe -> here; the block update with its
+// Gram V^T V):
+//                                    block update        W/P update     Gram P^T (A P) (in the product)
+//   27-point 96^3, KP = 16          1357 -> 258 + 66     408 -> 153      239 -> 131
+//   diffusion 64^3, KP = 32         1619 -> 283 + 116    471 -> 160      280 -> 126
+//   diffusion 100^3, KP = 8          455 -> 145 + 55     129 -> 88        78 -> 97 (kept fused)
+//   diffusion 128^3, KP = 4          288 -> 157 + 52      77 -> 92 (kept)  58 -> 110 (kept fused)
+// The same contractions in fixed point on the integer pipe (two 28-bit limbs, three IMAD.WIDE a term; 62
+// lanes per clock per SM) took 383 + 115 and 205 us at KP = 16. The tile shapes (16 rows, 16 columns at most) are those of mma.sync: a warp holds its operands
+// and results in registers in the layout in which it reads and writes them, so that there is no
+// staging, no shared memory but the k x k matrices' digits, and no barrier in the loops (tcgen05.mma's
+// smallest tile of 128 rows, with its operands in shared memory and results in tensor memory, needs
+// all of these).
+//
+// Digits. A group of values (a row of a block, a column of a k x k matrix, a column of the rows that a
+// warp sums) whose largest biased exponent is E is written x = 2^(E - 1022) 2^-B X, X the nearest
+// integer (|X| <= 2^B: the group's largest value keeps all its bits, any other loses what lies below
+// 2^-(B+1) of the scale), and X in 7 base-256 digits: six of -128..127 (X plus 128 in every digit, minus
+// 128 digit by digit) and a leading one of at most 2^(B-48), all exact in FP16. Digit pairs (t, u) are kept
+// for t + u <= 6 (28 products); what is dropped is random and below 2^-56 of the two scales at B = 56.
+// (With one side's digits 0..255, two operations fewer per pair of digits, what is dropped has a mean
+// that is the same for every row of a column: a smooth error, which an elliptic operator magnifies. The
+// state after 8 iterations of the 27-point stencil was 100 times further off.)
+//   A level sum S_L = sum_{t+u=L} sum_l is exact in the FP32 accumulator: below (2 * 2^15 + 5 * 2^14) * 16 <
+// 2^22 in the row products at B = 56, and 7 * 2^14 * 32 < 2^22 at the B = 55 of KP = 32; below 7 * 2^14 * 128
+// rows < 2^24 in a Gram (B = 55) between two drains.
+//
+// Widths. The row products see the block as rows of KV = max(KP, 8) columns and a Gram as rows of 16: for
+// a narrower block several rows make one, with the k x k matrix repeated on the diagonal (the diagonal
+// blocks of the Gram summed).
+//
+// A group that holds an infinity or a NaN has E = 0x7FF, and what is formed from it is NaN. A group below
+// 2^-958 counts as zero (the solver squares norms: it can use nothing below 2^-511).
+#pragma once
+#include <cuda_fp16.h>
+#include <stdint.h>
+
+#include <type_traits>
+
+#include "int_to_fp64.cuh"
+#include "mbpcg_device.cuh"
+
+namespace mbpcg {
+
+constexpr int kMxMinKP = 4;  // narrower blocks have too few FP64 operations per byte
+constexpr int kMxDigits = 7;
+constexpr int kMxThreads = 256;  // threads per CTA
+constexpr int kMxGramBits = 55;  // B of the Grams
+constexpr unsigned kMxAll = 0xffffffffu;
+
+__device__ __forceinline__ int mx_exponent(double x) { return (__double2hiint(x) >> 20) & 0x7FF; }
+
+// X of x in a group of scale exponent E (>= its own), to nearest (halves away from zero).
+template <int B>
+__device__ __forceinline__ long long mx_int(double x, int E) {
+  const int h = __double2hiint(x), e = (h >> 20) & 0x7FF;
+  // 53 bits moved up to B + 1 (one below the unit), then down to the group's scale;
+  // shr.u64 gives 0 from 64 on, which a zero or subnormal x (e = 0) reaches since E >= 64
+  const unsigned long long m = (((unsigned long long)(unsigned)((h & 0xFFFFF) | 0x100000) << 32) |
+                                (unsigned)__double2loint(x)) << (B - 52);
+  unsigned long long r;
+  asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(m), "r"((E < 64 ? 4096 : E) - e));
+  r = (r + 1) >> 1;
+  const long long s = h >> 31;
+  return (long long)(r ^ (unsigned long long)s) - s;
+}
+
+__device__ __forceinline__ uint32_t mx_prmt(uint32_t a, uint32_t b, uint32_t sel) {
+  uint32_t r;
+  asm("prmt.b32 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(b), "r"(sel));
+  return r;
+}
+// The 7 digits of the two integers a and b as FP16 pairs (a in the low half).
+__device__ __forceinline__ void mx_digits(long long a, long long b, uint32_t (&d)[kMxDigits]) {
+  constexpr long long kBias = 0x6600808080808080LL;  // 128 in every digit but the first, which becomes an FP16 1536 + d
+  const unsigned long long ua = (unsigned long long)(a + kBias), ub = (unsigned long long)(b + kBias);
+  const uint32_t w[3] = {mx_prmt((uint32_t)ua, (uint32_t)ub, 0x5140u), mx_prmt((uint32_t)ua, (uint32_t)ub, 0x7362u),
+                         mx_prmt((uint32_t)(ua >> 32), (uint32_t)(ub >> 32), 0x5140u)};
+  {
+    const uint32_t v = mx_prmt((uint32_t)(ua >> 32), (uint32_t)(ub >> 32), 0x7632u);
+    const __half2 r = __hsub2(*reinterpret_cast<const __half2*>(&v), __half2half2(__ushort_as_half(0x6600)));
+    d[0] = *reinterpret_cast<const uint32_t*>(&r);
+  }
+#pragma unroll
+  for (int t = 1; t < kMxDigits; ++t) {
+    const int byte = kMxDigits - 1 - t;
+    const uint32_t v = mx_prmt(w[byte >> 1], 0x64646464u, (byte & 1) ? 0x4342u : 0x4140u);  // 1024 + 128 + digit
+    const __half2 r = __hsub2(*reinterpret_cast<const __half2*>(&v), __half2half2(__ushort_as_half(0x6480)));
+    d[t] = *reinterpret_cast<const uint32_t*>(&r);
+  }
+}
+
+// D += A B, one warp: A 16 x 16 (or 16 x 8) by rows, B 16 x 8 (8 x 8) by columns, FP16 with FP32 sums.
+__device__ __forceinline__ void mx_mma16(float (&d)[4], const uint32_t* a, uint32_t b0, uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3},{%4,%5,%6,%7},{%8,%9},{%0,%1,%2,%3};"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ void mx_mma8(float (&d)[4], const uint32_t* a, uint32_t b0) {
+  asm("mma.sync.aligned.m16n8k8.row.col.f32.f16.f16.f32 {%0,%1,%2,%3},{%4,%5},{%6},{%0,%1,%2,%3};"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(b0));
+}
+
+// t 2^k as FP64, rounded to nearest (half up), by integer operations; below 2^-1022: zero.
+__device__ __forceinline__ double mx_double(long long t, int k) {
+  const int s = (int)(t >> 32) >> 31;
+  unsigned long long u = (unsigned long long)((t ^ (long long)s) - (long long)s);
+  int top = 1023 + 62 + k;  // exponent of bit 63, less one
+  if ((unsigned)(u >> 32) == 0) {  // rare, but for zeros (padded columns)
+    if (u == 0) return 0.0;
+    u <<= 32;
+    top -= 32;
+  }
+  const int lz = __clz((int)(u >> 32));
+  u <<= lz;
+  // the leading one of the rounded significand raises the exponent field by one, a carry by two
+  const unsigned long long m = (u >> 11) + ((u >> 10) & 1ull);
+  const int e = top - lz;
+  double v = __hiloint2double(((int)(m >> 32) + (e << 20)) | (s & (int)0x80000000), (int)m);
+  if (e < 0) v = 0.0;
+  if (e > 2044) v = __hiloint2double(0x7FF00000 | (s & (int)0x80000000), 0);
+  return v;
+}
+__device__ __forceinline__ double mx_nan() { return __hiloint2double(0x7FF80000, 0); }
+
+// ------------------------------------------------------------------------------------ row products
+
+// Widths of the row products: view rows of KV columns in NB blocks of 8; lane (g, t) = (lane / 4,
+// lane % 4) of a warp holds columns 8 c + 2 t, + 1 (c < NB) of the view rows g and g + 8 of its 16.
+template <int KP>
+struct MxRows {
+  static constexpr int KV = KP < 8 ? 8 : KP;
+  static constexpr int REP = KV / KP;  // rows of the block in a view row
+  static constexpr int NB = KV / 8;
+  static constexpr int KS = KV < 16 ? 1 : KV / 16;  // mma steps over the reduction index
+  static constexpr int B = KP >= 32 ? 55 : 56;
+};
+
+// A k x k matrix ready for the row products: the digits of each column in the fragment order of the
+// mma (one 8-byte load per lane), and the columns' scale exponents.
+template <int KP>
+struct MxMatrix {
+  using W = MxRows<KP>;
+  uint2 b[kMxDigits][W::KS][W::NB][32];
+  int e[KP];
+};
+
+// The accumulators of a row product start at 3 2^22, whose last bit is worth 1: their bits then count the
+// level sum, which stays below 2^22 (two mma steps of 2^21).
+constexpr uint32_t kMxStart = 0x4B400000u;
+
+// Weighted sum of the 7 levels' accumulators as integers, in units of 2^54 of the digits' product
+// (level L weighs 2^(8 (12 - L))), with the start values' share kMxStartSum, modulo 2^64: the total is
+// below 16 * 2^112 2^-54 = 2^62.
+__device__ __forceinline__ unsigned long long mx_levels(const float (&d)[kMxDigits][4], int q) {
+  unsigned long long r = __float_as_uint(d[6][q]) >> 6;
+  asm("mad.wide.u32 %0, %1, 4, %0;" : "+l"(r) : "r"(__float_as_uint(d[5][q])));
+  asm("mad.wide.u32 %0, %1, 1024, %0;" : "+l"(r) : "r"(__float_as_uint(d[4][q])));
+  asm("mad.wide.u32 %0, %1, 262144, %0;" : "+l"(r) : "r"(__float_as_uint(d[3][q])));
+  asm("mad.wide.u32 %0, %1, 67108864, %0;" : "+l"(r) : "r"(__float_as_uint(d[2][q])));
+  r += ((unsigned long long)((__float_as_uint(d[1][q]) << 2) + (__float_as_uint(d[0][q]) << 10))) << 32;
+  return r;
+}
+constexpr unsigned long long kMxStartSum =
+    (unsigned long long)(kMxStart >> 6) + (unsigned long long)kMxStart * (4ull + 1024ull + 262144ull + 67108864ull) +
+    ((unsigned long long)(uint32_t)((kMxStart << 2) + (kMxStart << 10)) << 32);
+
+// Fills M from src(l, j) (KP x KP; all threads; the caller synchronises before and after).
+template <int KP, typename F>
+__device__ void mx_load_matrix(F src, MxMatrix<KP>& M) {
+  using W = MxRows<KP>;
+  const int tid = threadIdx.x;
+  if (tid < KP) {
+    int e = 0;
+#pragma unroll 8
+    for (int l = 0; l < KP; ++l) e = max(e, mx_exponent(src(l, tid)));
+    M.e[tid] = e;
+  }
+  __syncthreads();
+  for (int q = tid; q < W::KS * W::NB * 32; q += kMxThreads) {
+    const int lane = q & 31, nb = (q >> 5) % W::NB, ks = (q >> 5) / W::NB;
+    const int n = 8 * nb + (lane >> 2), k0 = 16 * ks + 2 * (lane & 3);
+    // view matrix: KP x KP blocks on the diagonal
+    auto at = [&](int k) {
+      return (k < W::KV && k / KP == n / KP) ? mx_int<W::B>(src(k % KP, n % KP), M.e[n % KP]) : 0LL;
+    };
+    uint32_t d0[kMxDigits], d1[kMxDigits];
+    mx_digits(at(k0), at(k0 + 1), d0);
+    mx_digits(at(k0 + 8), at(k0 + 9), d1);
+#pragma unroll
+    for (int u = 0; u < kMxDigits; ++u) M.b[u][ks][nb][lane] = make_uint2(d0[u], d1[u]);
+  }
+}
+
+// A warp's 16 view rows of a block: digits, and the scale exponents of this lane's two rows.
+template <int KP>
+struct MxTile {
+  using W = MxRows<KP>;
+  uint32_t a[kMxDigits][2 * W::NB];
+  int e[2];
+
+  // v[c][r]: columns 8 c + 2 t, + 1 of view row g + 8 r
+  __device__ __forceinline__ void split(const double2 (&v)[W::NB][2]) {
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+      int m = 0;
+#pragma unroll
+      for (int c = 0; c < W::NB; ++c) m = max(m, max(mx_exponent(v[c][r].x), mx_exponent(v[c][r].y)));
+      m = max(m, __shfl_xor_sync(kMxAll, m, 1));
+      e[r] = max(m, __shfl_xor_sync(kMxAll, m, 2));
+#pragma unroll
+      for (int c = 0; c < W::NB; ++c) {
+        uint32_t d[kMxDigits];
+        mx_digits(mx_int<W::B>(v[c][r].x, e[r]), mx_int<W::B>(v[c][r].y, e[r]), d);
+#pragma unroll
+        for (int t = 0; t < kMxDigits; ++t) a[t][2 * c + r] = d[t];
+      }
+    }
+  }
+
+  // Columns 8 nb + 2 t, + 1 of the two rows times M: y[r].
+  __device__ __forceinline__ void times(const MxMatrix<KP>& M, int nb, double2 (&y)[2]) const {
+    const int lane = threadIdx.x & 31;
+    float d[kMxDigits][4];
+#pragma unroll
+    for (int L = 0; L < kMxDigits; ++L)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) d[L][q] = __uint_as_float(kMxStart);
+#pragma unroll
+    for (int ks = 0; ks < W::KS; ++ks)
+#pragma unroll
+      for (int u = 0; u < kMxDigits; ++u) {
+        const uint2 b = M.b[u][ks][nb][lane];
+#pragma unroll
+        for (int t = 0; t + u < kMxDigits; ++t) {
+          if constexpr (W::KV >= 16) mx_mma16(d[t + u], a[t] + 4 * ks, b.x, b.y);
+          else mx_mma8(d[t + u], a[t], b.x);
+        }
+      }
+    const int j = (8 * nb + 2 * (lane & 3)) % KP;
+    double v[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int f = M.e[j + (q & 1)], er = e[q >> 1];
+      v[q] = mx_double((long long)(mx_levels(d, q) - kMxStartSum), er + f - 2044 - 2 * W::B + 54);
+      if (max(f, er) == 0x7FF) v[q] = mx_nan();
+    }
+    y[0] = make_double2(v[0], v[1]);
+    y[1] = make_double2(v[2], v[3]);
+  }
+};
+
+// Loads v[c][r] from X, rows of the view up to nv (nf doubles in all: the last view row may be short).
+template <int KP>
+__device__ __forceinline__ void mx_load_rows(const double* X, size_t row, size_t nf, int t,
+                                             double2 (&v)[MxRows<KP>::NB][2]) {
+  using W = MxRows<KP>;
+#pragma unroll
+  for (int r = 0; r < 2; ++r)
+#pragma unroll
+    for (int c = 0; c < W::NB; ++c) {
+      const size_t o = (row + 8 * r) * W::KV + 8 * c + 2 * t;
+      v[c][r] = o < nf ? *reinterpret_cast<const double2*>(X + o) : make_double2(0.0, 0.0);
+    }
+}
+template <int KP>
+__device__ __forceinline__ void mx_store_rows(double* X, size_t row, size_t nf, int t,
+                                              const double2 (&v)[MxRows<KP>::NB][2]) {
+  using W = MxRows<KP>;
+#pragma unroll
+  for (int r = 0; r < 2; ++r)
+#pragma unroll
+    for (int c = 0; c < W::NB; ++c) {
+      const size_t o = (row + 8 * r) * W::KV + 8 * c + 2 * t;
+      if (o < nf) *reinterpret_cast<double2*>(X + o) = v[c][r];
+    }
+}
+
+// Block update of Algorithm 1 (as k_axpy): X~ += P T, R -= (A P) T, V = W - (A P) Xi, and the CTA partials
+// of nu at part[NPACK + j]. RFREE: R is neither read nor written, and there are no norms. Tiles of 16
+// view rows are dealt to the warps of the grid in turn (their sums do not depend on the order).
+template <int KP, bool RFREE>
+__global__ void __launch_bounds__(kMxThreads, KP >= 32 ? 1 : 2)
+k_axpy_mx(int n, const double* __restrict__ P, const double* __restrict__ Q, const double* __restrict__ W,
+          double* __restrict__ R, double* __restrict__ Xt, double* __restrict__ V, const double* __restrict__ Tg,
+          const double* __restrict__ Xig, const double* __restrict__ wdiag, double* __restrict__ part, int pstride,
+          const SolveState* __restrict__ st) {
+  using M = MxRows<KP>;
+  if (st->done) return;
+  __shared__ MxMatrix<KP> T, Xi;
+  __shared__ double red[RFREE ? 1 : kMxThreads / 32][KP];
+  mx_load_matrix<KP>([&](int l, int j) { return __ldg(Tg + l + j * KP); }, T);
+  mx_load_matrix<KP>([&](int l, int j) { return __ldg(Xig + l + j * KP); }, Xi);
+  __syncthreads();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
+  const size_t nf = (size_t)n * KP, nv = (nf + M::KV - 1) / M::KV;
+  const size_t step = (size_t)gridDim.x * (kMxThreads / 32) * 16;
+  double2 nu[M::NB];
+#pragma unroll
+  for (int c = 0; c < M::NB; ++c) nu[c] = make_double2(0.0, 0.0);
+  for (size_t base = ((size_t)blockIdx.x * (kMxThreads / 32) + warp) * 16; base < nv; base += step) {
+    const size_t row = base + g;
+    MxTile<KP> tile;
+    double2 v[M::NB][2], x[M::NB][2], y[2];
+    mx_load_rows<KP>(P, row, nf, t, v);
+    mx_load_rows<KP>(Xt, row, nf, t, x);
+    tile.split(v);
+    mx_load_rows<KP>(Q, row, nf, t, v);
+#pragma unroll
+    for (int c = 0; c < M::NB; ++c) {
+      tile.times(T, c, y);
+#pragma unroll
+      for (int r = 0; r < 2; ++r) {
+        x[c][r].x += y[r].x;
+        x[c][r].y += y[r].y;
+      }
+    }
+    mx_store_rows<KP>(Xt, row, nf, t, x);
+    mx_load_rows<KP>(W, row, nf, t, x);
+    tile.split(v);
+    if constexpr (!RFREE) mx_load_rows<KP>(R, row, nf, t, v);
+#pragma unroll
+    for (int c = 0; c < M::NB; ++c) {
+      tile.times(Xi, c, y);
+#pragma unroll
+      for (int r = 0; r < 2; ++r) {
+        x[c][r].x -= y[r].x;
+        x[c][r].y -= y[r].y;
+      }
+    }
+    mx_store_rows<KP>(V, row, nf, t, x);
+    if constexpr (!RFREE) {
+#pragma unroll
+      for (int c = 0; c < M::NB; ++c) {
+        tile.times(T, c, y);
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+          v[c][r].x -= y[r].x;
+          v[c][r].y -= y[r].y;
+          double wx = v[c][r].x, wy = v[c][r].y;
+          if (wdiag != nullptr) {
+            const size_t i = ((row + 8 * r) * M::KV + 8 * c + 2 * t) / KP;
+            const double w2 = i < (size_t)n ? __ldg(wdiag + i) : 0.0;
+            wx *= w2;
+            wy *= w2;
+          }
+          nu[c].x = fma(wx, v[c][r].x, nu[c].x);
+          nu[c].y = fma(wy, v[c][r].y, nu[c].y);
+        }
+      }
+      mx_store_rows<KP>(R, row, nf, t, v);
+    }
+  }
+  if constexpr (!RFREE) {  // lanes of one column, view columns of one column, then the warps in order
+#pragma unroll
+    for (int c = 0; c < M::NB; ++c) {
+#pragma unroll
+      for (int off = 16; off >= 4; off >>= 1) {
+        nu[c].x += __shfl_xor_sync(kMxAll, nu[c].x, off);
+        nu[c].y += __shfl_xor_sync(kMxAll, nu[c].y, off);
+      }
+      if constexpr (KP == 4) {
+        nu[c].x += __shfl_xor_sync(kMxAll, nu[c].x, 2);
+        nu[c].y += __shfl_xor_sync(kMxAll, nu[c].y, 2);
+      }
+      const int j = 8 * c + 2 * t;
+      if (g == 0 && j < KP) {
+        red[warp][j] = nu[c].x;
+        red[warp][j + 1] = nu[c].y;
+      }
+    }
+    __syncthreads();
+    if (threadIdx.x < KP) {
+      double a = red[0][threadIdx.x];
+      for (int w = 1; w < kMxThreads / 32; ++w) a += red[w][threadIdx.x];
+      part[(size_t)blockIdx.x * pstride + npack(KP) + threadIdx.x] = a;
+    }
+  }
+}
+
+// W/P update of Algorithm 1 (as k_pw): W = V zeta^{-1}, P = W + P zeta^T (SETP: P = W).
+template <int KP, bool SETP>
+__global__ void __launch_bounds__(kMxThreads, KP >= 32 ? 1 : 2)
+k_pw_mx(int n, const double* __restrict__ V, double* __restrict__ W, double* __restrict__ P,
+        const double* __restrict__ Zinvg, const double* __restrict__ Zg, const SolveState* __restrict__ st) {
+  using M = MxRows<KP>;
+  if (st != nullptr && st->pw_skip) return;
+  __shared__ MxMatrix<KP> Zi;
+  __shared__ typename std::conditional<SETP, int, MxMatrix<KP>>::type Zt;
+  mx_load_matrix<KP>([&](int l, int j) { return __ldg(Zinvg + l + j * KP); }, Zi);
+  if constexpr (!SETP) mx_load_matrix<KP>([&](int l, int j) { return __ldg(Zg + j + l * KP); }, Zt);
+  __syncthreads();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
+  const size_t nf = (size_t)n * KP, nv = (nf + M::KV - 1) / M::KV;
+  const size_t step = (size_t)gridDim.x * (kMxThreads / 32) * 16;
+  for (size_t base = ((size_t)blockIdx.x * (kMxThreads / 32) + warp) * 16; base < nv; base += step) {
+    const size_t row = base + g;
+    MxTile<KP> tile;
+    double2 v[M::NB][2], w[M::NB][2], y[2];
+    mx_load_rows<KP>(V, row, nf, t, v);
+    tile.split(v);
+    if constexpr (!SETP) mx_load_rows<KP>(P, row, nf, t, v);
+#pragma unroll
+    for (int c = 0; c < M::NB; ++c) tile.times(Zi, c, w[c]);
+    mx_store_rows<KP>(W, row, nf, t, w);
+    if constexpr (!SETP) {
+      tile.split(v);
+#pragma unroll
+      for (int c = 0; c < M::NB; ++c) {
+        tile.times(Zt, c, y);
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+          w[c][r].x += y[r].x;
+          w[c][r].y += y[r].y;
+        }
+      }
+    }
+    mx_store_rows<KP>(P, row, nf, t, w);
+  }
+}
+
+// ------------------------------------------------------------------------------------ Gram matrices
+
+// CTA partials of the upper triangle of X^T Y (Y = X when SYM), row i of X weighted by w_i when w is
+// given. A warp keeps its own column scales: the mma takes 16 view rows as its reduction index, so that a
+// lane holds the view columns g and g + 8 of 4 rows, as the left operand and as the right one alike. The
+// scales only grow; a tile that exceeds them (the first one, and then rarely: one bit of headroom) first
+// has the sums turned into FP64. KP = 32 is three problems of 16 columns (blockIdx.y: columns 0..15 with
+// themselves, with 16..31, and 16..31 with themselves).
+constexpr int kMxDrainTiles = 8;    // 128 rows between two drains of the FP32 sums into int64
+constexpr int kMxFlushTiles = 16;   // 256 rows of 2^54 between two conversions of the int64 sums
+
+template <int KP, bool SYM>
+__global__ void __launch_bounds__(kMxThreads, SYM && KP <= 16 ? 2 : 1)
+k_gram_mx(int n, const double* __restrict__ X, const double* __restrict__ Y, const double* __restrict__ w,
+          double* __restrict__ part, int pstride, const SolveState* __restrict__ st) {
+  constexpr int KV = 16, WARPS = kMxThreads / 32;
+  if (st != nullptr && st->done) return;
+  __shared__ double red[WARPS][KV * KV];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
+  // KP = 32: rows are 32 wide, this problem's columns start at xc (X) and yc (Y)
+  constexpr int LD = KP > KV ? KP : KV;
+  const int xc = KP > KV && blockIdx.y == 2 ? KV : 0, yc = KP > KV && blockIdx.y >= 1 ? KV : 0;
+  const size_t nf = (size_t)n * KP, nv = (nf + LD - 1) / LD;
+  const size_t step = (size_t)gridDim.x * WARPS * 16;
+
+  float acc[kMxDigits][2][4];
+  long long sum[2][4];
+  double f[2][4];
+  int ex[2] = {0, 0}, ey[2] = {0, 0};  // scale exponents of view columns g, g + 8
+  auto zero = [&]() {
+#pragma unroll
+    for (int L = 0; L < kMxDigits; ++L)
+#pragma unroll
+      for (int b = 0; b < 2; ++b)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[L][b][q] = 0.f;
+  };
+  // the FP32 sums into the int64 ones (units of 2^56 of the digits' product: level 5; level 6 rounded)
+  auto drain = [&]() {
+#pragma unroll
+    for (int b = 0; b < 2; ++b)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        int s[kMxDigits];
+#pragma unroll
+        for (int L = 0; L < kMxDigits; ++L) s[L] = __float2int_rn(acc[L][b][q]);
+        sum[b][q] += ((long long)s[0] << 40) + ((long long)s[1] << 32) + ((long long)s[2] << 24) +
+                     ((long long)s[3] << 16) + ((long long)s[4] << 8) + s[5] + ((s[6] + 128) >> 8);
+      }
+    zero();
+  };
+  // the int64 sums into FP64
+  auto flush = [&]() {
+#pragma unroll
+    for (int b = 0; b < 2; ++b)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        // entry (g + 8 (q / 2), 8 b + 2 t + q % 2)
+        const int el = ex[q >> 1];
+        const int ej = __shfl_sync(kMxAll, SYM && KP <= KV ? ex[b] : ey[b], (2 * t + (q & 1)) * 4);
+        bool ok;
+        const int k = el + ej - 2044 - 2 * kMxGramBits + 56;
+        double v = ll_to_double_scaled_rn(sum[b][q], k, ok);
+        if (!ok) v = ldexp(ll_to_double_rn(sum[b][q]), k);
+        f[b][q] += max(el, ej) == 0x7FF ? mx_nan() : v;
+        sum[b][q] = 0;
+      }
+  };
+  zero();
+#pragma unroll
+  for (int b = 0; b < 2; ++b)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      sum[b][q] = 0;
+      f[b][q] = 0.0;
+    }
+  // x[h][c]: row 2 t + (h & 1) + 8 (h >> 1) of the tile, view column g + 8 c
+  constexpr bool ONE = SYM && KP <= KV;  // both operands from one block
+  double x[4][2], y[ONE ? 1 : 4][2];
+  auto load = [&](size_t base) {
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+      const size_t r = base + 2 * t + (h & 1) + 8 * (h >> 1);
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        const size_t o = r * LD + g + 8 * c;
+        const bool in = r < nv && (KP >= KV || o < nf);
+        x[h][c] = in ? __ldg(X + o + xc) : 0.0;
+        if constexpr (!ONE) {
+          y[h][c] = in ? __ldg(Y + o + yc) : 0.0;
+          if (w != nullptr && in) x[h][c] *= __ldg(w + (o / KP));
+        }
+      }
+    }
+  };
+  auto grow = [&](const auto& v, int (&e)[2], int (&ne)[2]) {
+    bool over = false;
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      int m = max(max(mx_exponent(v[0][c]), mx_exponent(v[1][c])), max(mx_exponent(v[2][c]), mx_exponent(v[3][c])));
+      m = max(m, __shfl_xor_sync(kMxAll, m, 1));
+      m = max(m, __shfl_xor_sync(kMxAll, m, 2));
+      ne[c] = m > e[c] ? (m == 0x7FF ? m : min(m + 1, 0x7FE)) : e[c];
+      over |= ne[c] != e[c];
+    }
+    return over;
+  };
+  auto split = [&](const auto& v, const int (&e)[2], uint32_t (&a)[kMxDigits][4]) {
+#pragma unroll
+    for (int hh = 0; hh < 2; ++hh)
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        uint32_t d[kMxDigits];
+        mx_digits(mx_int<kMxGramBits>(v[2 * hh][c], e[c]), mx_int<kMxGramBits>(v[2 * hh + 1][c], e[c]), d);
+#pragma unroll
+        for (int q = 0; q < kMxDigits; ++q) a[q][2 * hh + c] = d[q];
+      }
+  };
+  int tiles = 0;
+  size_t base = ((size_t)blockIdx.x * WARPS + warp) * 16;
+  if (base < nv) load(base);
+  for (; base < nv; base += step) {
+    int nx[2], ny[2];
+    bool over = grow(x, ex, nx);
+    if constexpr (!ONE) over |= grow(y, ey, ny);
+    if (__any_sync(kMxAll, over)) {
+      drain();
+      flush();
+      tiles = 0;
+      ex[0] = nx[0];
+      ex[1] = nx[1];
+      if constexpr (!ONE) {
+        ey[0] = ny[0];
+        ey[1] = ny[1];
+      }
+    }
+    uint32_t a[kMxDigits][4], b[ONE ? 1 : kMxDigits][4];
+    split(x, ex, a);
+    if constexpr (!ONE) split(y, ey, b);
+    if (base + step < nv) load(base + step);
+#pragma unroll
+    for (int u = 0; u < kMxDigits; ++u) {
+      const uint32_t* bu = ONE ? a[u] : b[ONE ? 0 : u];
+#pragma unroll
+      for (int q = 0; q + u < kMxDigits; ++q) {
+        mx_mma16(acc[q + u][0], a[q], bu[0], bu[2]);
+        mx_mma16(acc[q + u][1], a[q], bu[1], bu[3]);
+      }
+    }
+    ++tiles;
+    if (tiles % kMxDrainTiles == 0) drain();
+    if (tiles == kMxFlushTiles) {
+      flush();
+      tiles = 0;
+    }
+  }
+  drain();
+  flush();
+#pragma unroll
+  for (int b = 0; b < 2; ++b)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) red[warp][(g + 8 * (q >> 1)) * KV + 8 * b + 2 * t + (q & 1)] = f[b][q];
+  __syncthreads();
+  double* out = part + (size_t)blockIdx.x * pstride;
+  constexpr int KB = KP < KV ? KP : KV;  // the diagonal blocks are KB wide
+  for (int q = threadIdx.x; q < KB * KB; q += kMxThreads) {
+    const int l = q / KB, j = q % KB;
+    const int L = l + xc, J = j + yc;
+    if (L > J) continue;
+    double v = 0.0;
+    for (int d = 0; d < KV / KB; ++d)
+      for (int k = 0; k < WARPS; ++k) v += red[k][(l + d * KB) * KV + j + d * KB];
+    out[pidx(L, J)] = v;
+  }
+}
+
+}  // namespace mbpcg
