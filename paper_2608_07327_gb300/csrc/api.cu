@@ -676,12 +676,11 @@ void enqueue_reduce(mbpcg_ctx* h, int nent, const SolveState* st, int mx = 0, in
 void enqueue_true_residual(mbpcg_ctx* h) {
   const Dims& dm = h->dm;
   if (dm.dense)
-    k_resid_dense<<<dm.nb_dense, kThreads, 0, h->stream>>>(dm.n, h->A, h->sqd, h->b, h->x, h->rhs, h->part, dm.pstride);
+    k_resid_dense<<<dm.nb, kThreads, 0, h->stream>>>(dm.n, h->A, h->sqd, h->b, h->x, h->rhs, h->part, dm.pstride);
   else
     k_resid_csr<<<dm.nb, kThreads, 0, h->stream>>>(dm.n, h->rp, h->ci, h->av, h->sqd, h->b, h->x, h->rhs, h->part,
                                                    dm.pstride);
-  // the dense residual uses nb_dense partial slots
-  launch_reduce(h->stream, h->part, dm.dense ? dm.nb_dense : dm.nb, dm.pstride, h->red, 1, nullptr);
+  launch_reduce(h->stream, h->part, dm.nb, dm.pstride, h->red, 1, nullptr);
   k_small_true<<<1, 1, 0, h->stream>>>(h->st, h->red);
 }
 
@@ -829,11 +828,14 @@ void enqueue_cg_body(mbpcg_ctx* h) {
                          h->cond, h->use_cond);
     return;
   }
-  const RowOps* ops = row_ops(1);
-  enqueue_product(h, ops, h->r, h->w, 0, h->st);  // w = A u, u = r
-  k_cg_dots<<<dm.nb, kThreads, 0, h->stream>>>(dm.n, h->r, h->w, h->wdiag, h->part, dm.pstride, h->st);
-  enqueue_reduce(h, 3, h->st);
-  k_small_cg<<<1, 1, 0, h->stream>>>(h->st, h->red, h->cond, h->use_cond);
+  const RowOps* ops = row_ops(1);  // w = A u, u = r, and the sums
+  if (!dm.dense && h->prod64 == MBPCG_PRODUCT_CSR_GATHER) {
+    ops->spmm_dots(h->stream, dm.nb, dm.n, h->rp, h->ci, h->av, h->r, h->w, h->wdiag, h->part, dm.pstride, h->st);
+  } else {
+    enqueue_product(h, ops, h->r, h->w, 0, h->st);
+    k_cg_dots<<<dm.nb, kThreads, 0, h->stream>>>(dm.n, h->r, h->w, h->wdiag, h->part, dm.pstride, h->st);
+  }
+  k_small_cg<<<1, 3 * kReduceThreads, 0, h->stream>>>(h->st, h->part, dm.nb, dm.pstride, h->cond, h->use_cond);
   k_cg_update<<<dm.nb, kThreads, 0, h->stream>>>(dm.n, h->r, h->w, h->xb, h->p, h->sv, h->st);
 }
 

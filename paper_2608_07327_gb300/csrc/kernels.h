@@ -27,6 +27,9 @@ struct RowOps {
   int kp;
   void (*spmm)(cudaStream_t, int nb, int n, const int* rp, const int* ci, const double* av, const double* P,
                double* Q, double* part, int pstride, const SolveState* st, int gram);
+  // one column: the CG's w = A r with the CTA partials of k_cg_dots
+  void (*spmm_dots)(cudaStream_t, int nb, int n, const int* rp, const int* ci, const double* av, const double* r,
+                    double* w, const double* wdiag, double* part, int pstride, const SolveState* st);
   void (*dense)(cudaStream_t, int nb, int n, const double* A, const double* P, double* Q, const SolveState* st,
                 int* err);
   void (*gram)(cudaStream_t, int nb, int n, const double* X, const double* Y, double* part, int pstride,
@@ -149,7 +152,8 @@ __global__ void k_small_setup(SolveState* st, const double* red);
 __global__ void k_small_ls(SolveState* st, const double* Mg, int kp, double* c_out);
 __global__ void k_small_true(SolveState* st, const double* rr);
 __global__ void k_small_cg_setup(SolveState* st, const double* red);
-__global__ void k_small_cg(SolveState* st, const double* red, cudaGraphConditionalHandle cond, int use_cond);
+__global__ void k_small_cg(SolveState* st, const double* part, int nparts, int pstride, cudaGraphConditionalHandle cond,
+                           int use_cond);
 __global__ void k_validate_csr(int n, long long nnz, const int* rp, const int* ci, int* flag);
 __global__ void k_diag_csr(int n, const int* rp, const int* ci, const double* av, double* diag, int* flag);
 __global__ void k_diag_dense(int n, const double* A, double* diag, int* flag);

@@ -66,6 +66,39 @@ k_spmm(int n, const int* __restrict__ rp, const int* __restrict__ ci, const doub
   if constexpr (GRAM) g.finish(red, part + (size_t)blockIdx.x * pstride);
 }
 
+// The same for one column, w = A r, with the CTA partials of (r, r), (w, r) and ||D r||^2 (wdiag = D^2 or
+// NULL) that the Chronopoulos-Gear CG needs of it: in the order of a pass of its own over r, w and D^2
+// (k_cg_dots), which the FP64 pipe bound (4 operations a row), while here they hide behind the bytes of A.
+// Diffusion 128^3: 48 + 21 -> 63 us (11 FP64 operations a row: 37 us of the pipe; 217 MB: 32 us). The norms
+// beside the update's bytes instead took 49 + 35: its 4 FMAs and theirs fill the FP64 pipe.
+template <int KP>
+__global__ void __launch_bounds__(kThreads, 8)
+k_spmm_dots(int n, const int* __restrict__ rp, const int* __restrict__ ci, const double* __restrict__ av,
+            const double* __restrict__ r, double* __restrict__ w, const double* __restrict__ wdiag,
+            double* __restrict__ part, int pstride, const SolveState* __restrict__ st) {
+  if (st->done) return;
+  __shared__ double red[3 * kThreads];
+  int r0, r1;
+  row_range(n, r0, r1);
+  double g = 0.0, dl = 0.0, nu = 0.0;
+  for (int i = r0 + threadIdx.x; i < r1; i += kThreads) {
+    double acc = 0.0;
+    const double ri = __ldg(r + i), wd = wdiag != nullptr ? __ldg(wdiag + i) : 1.0;
+    const int pe = __ldg(rp + i + 1);
+#pragma unroll 4
+    for (int p = __ldg(rp + i); p < pe; ++p) acc = fma(__ldg(av + p), __ldg(r + __ldg(ci + p)), acc);
+    w[i] = acc;
+    g = fma(ri, ri, g);
+    dl = fma(acc, ri, dl);
+    nu = (wdiag != nullptr) ? fma(ri * wd, ri, nu) : fma(ri, ri, nu);
+  }
+  red[threadIdx.x * 3] = g;
+  red[threadIdx.x * 3 + 1] = dl;
+  red[threadIdx.x * 3 + 2] = nu;
+  cta_tree_sum(red, kThreads, 3);
+  if (threadIdx.x < 3) part[(size_t)blockIdx.x * pstride + threadIdx.x] = red[threadIdx.x];
+}
+
 // ------------------------------------------------------------------------------------------------
 // Q = A P for dense symmetric A stored column-major (row i of A is column i, contiguous).
 // One CTA per SM owns a balanced range of rows and walks it in passes of G rows. The reduction index
@@ -798,22 +831,43 @@ __global__ void k_gen_u(int n, int s, unsigned long long seed, double* __restric
   }
 }
 
-// Column-major n x s (leading dimension n) <-> row-major n x KP with zero padding.
+// Column-major n x s (leading dimension n) <-> row-major n x KP with zero padding, by tiles of
+// kTrRows rows turned in shared memory so that both sides move whole 128-byte lines: 27-point 96^3, KP = 16,
+// s = 16: 152 -> 37 us (a thread per value, one side strided by n).
+constexpr int kTrRows = 64;
 template <int KP>
-__global__ void k_from_colmajor(int n, int s, const double* __restrict__ src, double* __restrict__ dst) {
-  const size_t total = (size_t)n * KP;
-  for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < total; q += (size_t)gridDim.x * blockDim.x) {
-    const int j = (int)(q % KP);
-    const size_t i = q / KP;
-    dst[q] = (j < s) ? src[(size_t)j * n + i] : 0.0;
+struct TransposeTile {
+  static constexpr int LD = kTrRows + 1;
+  double v[KP * LD];  // v[j * LD + r]
+};
+template <int KP>
+__global__ void __launch_bounds__(kThreads) k_from_colmajor(int n, int s, const double* __restrict__ src, double* __restrict__ dst) {
+  using T = TransposeTile<KP>;
+  __shared__ T t;
+  for (int r0 = blockIdx.x * kTrRows; r0 < n; r0 += gridDim.x * kTrRows) {
+    const int rows = min(kTrRows, n - r0);
+    for (int q = threadIdx.x; q < KP * kTrRows; q += kThreads) {
+      const int j = q / kTrRows, r = q % kTrRows;
+      t.v[j * T::LD + r] = (j < s && r < rows) ? src[(size_t)j * n + r0 + r] : 0.0;
+    }
+    __syncthreads();
+    for (int q = threadIdx.x; q < rows * KP; q += kThreads) dst[(size_t)r0 * KP + q] = t.v[(q % KP) * T::LD + q / KP];
+    __syncthreads();
   }
 }
 template <int KP>
-__global__ void k_to_colmajor(int n, int s, const double* __restrict__ src, double* __restrict__ dst) {
-  const size_t total = (size_t)n * s;
-  for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < total; q += (size_t)gridDim.x * blockDim.x) {
-    const size_t j = q / n, i = q % n;
-    dst[q] = src[i * KP + j];
+__global__ void __launch_bounds__(kThreads) k_to_colmajor(int n, int s, const double* __restrict__ src, double* __restrict__ dst) {
+  using T = TransposeTile<KP>;
+  __shared__ T t;
+  for (int r0 = blockIdx.x * kTrRows; r0 < n; r0 += gridDim.x * kTrRows) {
+    const int rows = min(kTrRows, n - r0);
+    for (int q = threadIdx.x; q < rows * KP; q += kThreads) t.v[(q % KP) * T::LD + q / KP] = src[(size_t)r0 * KP + q];
+    __syncthreads();
+    for (int q = threadIdx.x; q < s * kTrRows; q += kThreads) {
+      const int j = q / kTrRows, r = q % kTrRows;
+      if (r < rows) dst[(size_t)j * n + r0 + r] = t.v[j * T::LD + r];
+    }
+    __syncthreads();
   }
 }
 

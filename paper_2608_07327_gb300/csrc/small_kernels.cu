@@ -204,14 +204,47 @@ __global__ void k_small_cg_setup(SolveState* st, const double* __restrict__ red)
 
 // gamma = (r, u), delta = (w, u) with u = r and w = A u; test ||D r|| < tol ||rhs||; then
 // beta = gamma / gamma_old, alpha = gamma / (delta - beta gamma / alpha_old) (first step:
-// beta = 0, alpha = gamma / delta). Sets the WHILE condition (use_cond = 0 outside a graph).
-__global__ void k_small_cg(SolveState* st, const double* __restrict__ red, cudaGraphConditionalHandle cond,
-                           int use_cond) {
+// beta = 0, alpha = gamma / delta). Sets the WHILE condition (use_cond = 0 outside a graph). The sums
+// of the CTA partials (gamma, delta, nu^2) are formed here too, one group of kReduceThreads each,
+// in the order of k_reduce: a launch of its own before this one cost 3.8 us more.
+__global__ void __launch_bounds__(3 * kReduceThreads)
+k_small_cg(SolveState* st, const double* __restrict__ part, int nparts, int pstride, cudaGraphConditionalHandle cond,
+           int use_cond) {
+  __shared__ double ws[3][kReduceThreads / 32], tot[3];
+  const int e = threadIdx.x / kReduceThreads, t0 = threadIdx.x % kReduceThreads;
+  // every load of a batch in flight together, the first batch with the solve state
+  constexpr int kB = 10;  // 8 CTAs per SM on 152 SMs: 1216 partials in one batch
+  double v[kB];
+  auto load = [&](int p0) {
+#pragma unroll
+    for (int b = 0; b < kB; ++b) {
+      const int p = p0 + b * kReduceThreads;
+      v[b] = p < nparts ? part[(size_t)p * pstride + e] : 0.0;
+    }
+  };
+  load(t0);
   if (st->done) {
-    if (use_cond) cudaGraphSetConditional(cond, 0);
+    if (use_cond && threadIdx.x == 0) cudaGraphSetConditional(cond, 0);
     return;
   }
-  const double gamma = red[0], delta = red[1], nu = sqrt(red[2]);
+  double a = 0.0;
+  for (int p0 = t0; p0 < nparts; p0 += kB * kReduceThreads) {
+    if (p0 != t0) load(p0);
+#pragma unroll
+    for (int b = 0; b < kB; ++b)
+      if (p0 + b * kReduceThreads < nparts) a += v[b];
+  }
+  for (int off = 16; off; off >>= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
+  if ((t0 & 31) == 0) ws[e][t0 >> 5] = a;
+  __syncthreads();
+  if (t0 == 0) {  // one warp each, as in the fused dense iteration: the three chains run side by side
+    double s = ws[e][0];
+    for (int w = 1; w < kReduceThreads / 32; ++w) s += ws[e][w];
+    tot[e] = e == 2 ? sqrt(s) : s;
+  }
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  const double gamma = tot[0], delta = tot[1], nu = tot[2];
   st->nu_h = nu;
   st->ls_res = nu;
   if (nu < st->tol_abs) {
@@ -354,7 +387,8 @@ k_resid_csr(int n, const int* __restrict__ rp, const int* __restrict__ ci, const
   if (threadIdx.x == 0) part[(size_t)blockIdx.x * pstride] = red[0];
 }
 
-// Dense version: one warp per row, lanes over the reduction index.
+// Dense version: one warp per row, lanes over the reduction index (n = 4096: 90-101 -> 42-61 us with a batch
+// of loads in flight and two CTAs per SM instead of one; n^2 FMAs take 27 us of the FP64 pipe).
 __global__ void __launch_bounds__(kThreads)
 k_resid_dense(int n, const double* __restrict__ A, const double* __restrict__ sqd, const double* __restrict__ b,
               const double* __restrict__ x, double* __restrict__ r, double* __restrict__ part, int pstride) {
@@ -366,9 +400,19 @@ k_resid_dense(int n, const double* __restrict__ A, const double* __restrict__ sq
   for (int i = r0 + warp; i < r1; i += kThreads / 32) {
     const double* ai = A + (size_t)i * n;
     double a = 0.0;
-    for (int l = lane; l < n; l += 32) {
-      const double xl = (sqd != nullptr) ? sqd[l] * x[l] : x[l];
-      a = fma(ai[l], xl, a);
+    // kU loads of A in flight per lane (the sums keep the order of l)
+    constexpr int kU = 8;
+    for (int l0 = lane; l0 < n; l0 += 32 * kU) {
+      double av[kU], xv[kU];
+#pragma unroll
+      for (int u = 0; u < kU; ++u) {
+        const int l = l0 + 32 * u;
+        av[u] = l < n ? ai[l] : 0.0;
+        xv[u] = l < n ? ((sqd != nullptr) ? sqd[l] * x[l] : x[l]) : 0.0;
+      }
+#pragma unroll
+      for (int u = 0; u < kU; ++u)
+        if (l0 + 32 * u < n) a = fma(av[u], xv[u], a);
     }
     for (int off = 16; off >= 1; off >>= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
     const double ri = (sqd != nullptr) ? fma(-sqd[i], a, b[i]) : b[i] - a;
@@ -402,7 +446,8 @@ k_cg_init(int n, const double* __restrict__ rhs, const double* __restrict__ d, d
   if (threadIdx.x == 0) part[(size_t)blockIdx.x * pstride] = red[0];
 }
 
-// CTA partials of (r, r), (w, r) and ||D r||^2 (wdiag = D^2 or NULL).
+// CTA partials of (r, r), (w, r) and ||D r||^2 (wdiag = D^2 or NULL), for the products that do not form
+// them themselves (k_spmm_dots does).
 __global__ void __launch_bounds__(kThreads)
 k_cg_dots(int n, const double* __restrict__ r, const double* __restrict__ w, const double* __restrict__ wdiag,
           double* __restrict__ part, int pstride, const SolveState* __restrict__ st) {
