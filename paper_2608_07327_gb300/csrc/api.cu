@@ -6,6 +6,7 @@
 // the loop condition), and the exit kernels (least-squares combination, x update, true residual).
 // The host only reads the 200-byte solve state after each launch to decide on a true-residual
 // restart.
+#include <algorithm>
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
@@ -1504,9 +1505,11 @@ int32_t mbpcg_k_padded_width(int32_t s) { return (s >= 1 && s <= 32) ? padded_wi
 
 size_t mbpcg_k_scratch_bytes(int32_t n, int32_t s) {
   if (n < 1 || s < 1 || s > 32) return 0;
-  Dims dm = make_dims(n, 0, s, MBPCG_ALGO_MBPCG, 0, num_sms());
-  apply_mixed(dm);  // enough partial slots for the FP64 and the FP32 launch configurations
-  return (size_t)(dm.nbmax + 1) * dm.pstride * sizeof(double);
+  // slots for the FP64 and the FP32 launch configurations; the FP64 one has more CTAs at KP = 32 (8 rows
+  // each) and the CSR one at least as many as the dense one
+  Dims dm = make_dims(n, 0, s, MBPCG_ALGO_MBPCG, 0, num_sms()), df = dm;
+  apply_mixed(df);
+  return (size_t)(std::max(dm.nbmax, df.nbmax) + 1) * dm.pstride * sizeof(double);
 }
 
 static int k_product_gram(int dense, int32_t n, const int32_t* rp, const int32_t* ci, const double* av,
