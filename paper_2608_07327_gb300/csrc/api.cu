@@ -46,6 +46,7 @@ constexpr int kMixedRestarts = 12;       // refinement steps of the mixed-precis
 constexpr int kTuneVariants = 11;        // FP32 A P launch shapes tried by the autotuner
 constexpr int kTiledMinRows = 65536;     // smaller systems sit in L2 and keep the gather kernel
 constexpr double kMixedInnerTol = 1e-5;  // smallest relative tolerance asked of an FP32 inner solve
+constexpr int kLoopIters = 64;          // iterations per launch of the one-cluster loop
 constexpr int kBodyUnroll = 8;           // loop iterations per pass of the graph's WHILE node
 inline size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 // Runs of staged rows the workspace holds for a CSR plan (a stencil needs a few per tile; a
@@ -275,6 +276,8 @@ struct mbpcg_ctx {
   SpmmPlan plan;    // CSR: rows of P staged per tile (see spmm_tiled.cu)
   int use_tiled;    // 1: the matrix has a tiling plan
   int plan_tried;   // 1: build_plan has run (a plan is built at most once)
+  int loop_cl;      // the loop may run in one cluster (loop_cluster.cu)
+  int loop_slice;   // ... and its slice of A
   int prod64;       // the FP64 CSR product kernel: MBPCG_PRODUCT_CSR_GATHER or _TILED
   int round_once;   // tensor-core product: MBPCG_ROUND_ONCE (levels 5..8 exact) instead of the FP32 carry
   float spmm64_us[2];  // the FP64 product at create: gather and tiled kernels (0: not timed)
@@ -634,6 +637,12 @@ int finish_create(mbpcg_ctx* h) {
     h->prod64 = MBPCG_PRODUCT_CSR_GATHER;
     int rc = time_spmm64(h, MBPCG_PRODUCT_CSR_GATHER);
     if (rc) return rc;
+    if (h->algo == MBPCG_ALGO_MBPCG && loop_cluster_fits(h->dm.kp, n, h->dm.nnz)) {
+      loop_cluster_slice(h->stream, n, h->rp, h->flag);
+      CUDA_TRY(cudaGetLastError());
+      if ((rc = read_flag(h, &h->loop_slice))) return rc;
+      h->loop_cl = loop_cluster_ready(h->dm.kp, n, h->loop_slice);
+    }
   }
   if (h->dm.cg_fused) CUDA_TRY(cg_dense_configure(n, h->dm.nb_cg));
   if (h->dm.tc) {
@@ -701,10 +710,20 @@ void enqueue_mbpcg_setup(mbpcg_ctx* h) {
   else ops->pw(h->stream, dm.nb, n, h->R, h->W, h->P, h->SigmaInv, nullptr, nullptr, 1, dm.tc ? h->oz_ep : nullptr);
 }
 
+// A small CSR system iterates in one cluster, unless the residual is implicit or the tiled product imposed.
+bool in_loop_cluster(const mbpcg_ctx* h) {
+  return h->loop_cl && !h->rfree && h->prod64 == MBPCG_PRODUCT_CSR_GATHER;
+}
+
 void enqueue_mbpcg_body(mbpcg_ctx* h) {
   const Dims& dm = h->dm;
   const RowOps* ops = row_ops(dm.kp);
   const int kp = dm.kp, n = dm.n;
+  if (in_loop_cluster(h)) {
+    const LoopArgs a = {n, h->loop_slice, h->rp, h->ci, h->av, h->Xt, h->R, h->W, h->P, h->wdiag, h->Sigma, h->st};
+    launch_loop_cluster(h->stream, kp, a, h->use_cond ? kLoopIters : 1, h->cond, h->use_cond);
+    return;
+  }
   // tensor-core handles at KP >= 16: the k x k-row products of the two row passes on the tensor cores
   const bool tcrows = h->rp3 != nullptr && !h->rfree;
   double *Y0 = h->rp3, *Y1 = Y0 + (size_t)n * kp, *Y2 = Y1 + (size_t)n * kp;
@@ -891,7 +910,7 @@ cudaError_t capture_solve(mbpcg_ctx* h, cudaGraph_t g, cudaGraphConditionalHandl
         // this GPU, on top of ~1 us per kernel; every loop kernel returns at once after the
         // iteration in which the solve stopped, and the last one of a pass sets the condition
         h->use_cond = 1;
-        for (int u = 0; u < kBodyUnroll; ++u) {
+        for (int u = 0; u < (in_loop_cluster(h) ? 1 : kBodyUnroll); ++u) {
           if (cg) enqueue_cg_body(h);
           else if (h->dm.mixed) enqueue_mbpcg_body_f(h);
           else enqueue_mbpcg_body(h);

@@ -221,6 +221,22 @@ void launch_cg_dense_iter(cudaStream_t s, int nb, int n, const double* A, const 
                           double* part, int pstride, unsigned int* counter, SolveState* st,
                           cudaGraphConditionalHandle cond, int use_cond);
 
+// The iteration loop of a small CSR system in one launch of one thread-block cluster (loop_cluster.cu).
+struct LoopArgs {
+  int n, slice;  // slice: entries of A in the largest of the CTAs' row ranges (loop_cluster_slice)
+  const int *rp, *ci;
+  const double* av;
+  double *X, *R, *W, *P;
+  const double* wdiag;
+  double* Sigma;
+  SolveState* st;
+};
+bool loop_cluster_fits(int kp, int n, long long nnz);  // the sizes it is for
+void loop_cluster_slice(cudaStream_t s, int n, const int* rp, int* out);
+bool loop_cluster_ready(int kp, int n, int slice);  // it fits in shared memory and the device can schedule it
+void launch_loop_cluster(cudaStream_t s, int kp, const LoopArgs& a, int iters, cudaGraphConditionalHandle cond,
+                         int use_cond);
+
 // FP32 dense product of the mixed-precision inner solve (dense_f32.cu): Q = A P with A in the FP32
 // tiles k_dense_to_f32_tiles writes (dense_f32_tiles_bytes(n) bytes), P and Q row-major n x kp;
 // st may be NULL.
