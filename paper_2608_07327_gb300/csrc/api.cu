@@ -277,7 +277,7 @@ struct mbpcg_ctx {
   int use_tiled;    // 1: the matrix has a tiling plan
   int plan_tried;   // 1: build_plan has run (a plan is built at most once)
   int loop_cl;      // the loop may run in one cluster (loop_cluster.cu)
-  int loop_slice;   // ... and its slice of A
+  int loop_zcap;    // ... with so many entries of A in each CTA's shared memory
   int prod64;       // the FP64 CSR product kernel: MBPCG_PRODUCT_CSR_GATHER or _TILED
   int round_once;   // tensor-core product: MBPCG_ROUND_ONCE (levels 5..8 exact) instead of the FP32 carry
   float spmm64_us[2];  // the FP64 product at create: gather and tiled kernels (0: not timed)
@@ -640,8 +640,10 @@ int finish_create(mbpcg_ctx* h) {
     if (h->algo == MBPCG_ALGO_MBPCG && loop_cluster_fits(h->dm.kp, n, h->dm.nnz)) {
       loop_cluster_slice(h->stream, n, h->rp, h->flag);
       CUDA_TRY(cudaGetLastError());
-      if ((rc = read_flag(h, &h->loop_slice))) return rc;
-      h->loop_cl = loop_cluster_ready(h->dm.kp, n, h->loop_slice);
+      int slice = 0;
+      if ((rc = read_flag(h, &slice))) return rc;
+      h->loop_zcap = loop_cluster_ready(h->dm.kp, n, slice);
+      h->loop_cl = h->loop_zcap >= 0;
     }
   }
   if (h->dm.cg_fused) CUDA_TRY(cg_dense_configure(n, h->dm.nb_cg));
@@ -720,7 +722,7 @@ void enqueue_mbpcg_body(mbpcg_ctx* h) {
   const RowOps* ops = row_ops(dm.kp);
   const int kp = dm.kp, n = dm.n;
   if (in_loop_cluster(h)) {
-    const LoopArgs a = {n, h->loop_slice, h->rp, h->ci, h->av, h->Xt, h->R, h->W, h->P, h->wdiag, h->Sigma, h->st};
+    const LoopArgs a = {n, h->loop_zcap, h->rp, h->ci, h->av, h->Xt, h->R, h->W, h->P, h->wdiag, h->Sigma, h->st};
     launch_loop_cluster(h->stream, kp, a, h->use_cond ? kLoopIters : 1, h->cond, h->use_cond);
     return;
   }

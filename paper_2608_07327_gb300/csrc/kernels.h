@@ -223,7 +223,7 @@ void launch_cg_dense_iter(cudaStream_t s, int nb, int n, const double* A, const 
 
 // The iteration loop of a small CSR system in one launch of one thread-block cluster (loop_cluster.cu).
 struct LoopArgs {
-  int n, slice;  // slice: entries of A in the largest of the CTAs' row ranges (loop_cluster_slice)
+  int n, zcap;  // zcap: entries of A that a CTA keeps in shared memory (loop_cluster_ready)
   const int *rp, *ci;
   const double* av;
   double *X, *R, *W, *P;
@@ -233,7 +233,9 @@ struct LoopArgs {
 };
 bool loop_cluster_fits(int kp, int n, long long nnz);  // the sizes it is for
 void loop_cluster_slice(cudaStream_t s, int n, const int* rp, int* out);
-bool loop_cluster_ready(int kp, int n, int slice);  // it fits in shared memory and the device can schedule it
+// -1 unless the blocks fit in shared memory and the device can schedule the cluster; slice: entries of A in
+// the largest of the CTAs' row ranges (loop_cluster_slice)
+int loop_cluster_ready(int kp, int n, int slice);
 void launch_loop_cluster(cudaStream_t s, int kp, const LoopArgs& a, int iters, cudaGraphConditionalHandle cond,
                          int use_cond);
 

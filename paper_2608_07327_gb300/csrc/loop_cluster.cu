@@ -21,6 +21,7 @@
 // the additions of the sums (16.5 us).
 #include <cooperative_groups.h>
 
+#include <algorithm>
 #include <cfloat>
 
 #include "kernels.h"
@@ -308,7 +309,7 @@ template <int KP>
 __global__ void __launch_bounds__(kLcThreads, 1)
 k_loop_cluster(int n, const int* __restrict__ rp, const int* __restrict__ ci, const double* __restrict__ av,
                double* Xg, double* Rg, double* Wg, double* Pg, const double* __restrict__ wdiag, double* Sigma,
-               SolveState* st, int iters, cudaGraphConditionalHandle cond, int use_cond) {
+               SolveState* st, int zcap, int iters, cudaGraphConditionalHandle cond, int use_cond) {
   using C = LcCfg<KP>;
   extern __shared__ __align__(16) double blocks[];
   __shared__ LcShared<KP> sm;
@@ -328,18 +329,21 @@ k_loop_cluster(int n, const int* __restrict__ rp, const int* __restrict__ ci, co
   const int r0 = (int)((long long)n * rank / kLcCtas), r1 = (int)((long long)n * (rank + 1) / kLcCtas);
   const int tot = (r1 - r0) * KP, cap = ((n + kLcCtas - 1) / kLcCtas * KP + 1) & ~1;
   double *X = blocks, *R = X + cap, *W = R + cap, *P = W + cap, *Q = P + cap, *V = Q + cap;
-  // the CTA's rows of A: values, the address of P's row in the CTA that owns it, row starts
+  // the CTA's rows of A, the first zcap entries of them: values, the address of P's row in the CTA that owns
+  // it; row starts
   const int p0 = __ldg(rp + r0), nz = __ldg(rp + r1) - p0;
   double* as = V + cap;
-  uint32_t* ps = reinterpret_cast<uint32_t*>(as + nz);
-  int* rs = reinterpret_cast<int*>(ps + nz);
+  uint32_t* ps = reinterpret_cast<uint32_t*>(as + zcap);
+  int* rs = reinterpret_cast<int*>(ps + zcap);
   const uint32_t pbase = (uint32_t)__cvta_generic_to_shared(P);
-  for (int p = tid; p < nz; p += kLcThreads) {
-    const int col = __ldg(ci + p0 + p);
-    const int own = (int)((16LL * col + 15) / n);  // the last CTA whose first row is not after col
+  auto p_row = [&](int col) {
+    const int own = (int)((unsigned)(kLcCtas * col + kLcCtas - 1) / (unsigned)n);  // the CTA whose rows have col
     uint32_t a;
     asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(pbase), "r"(own));
-    ps[p] = a + (uint32_t)(col - (int)((long long)n * own / kLcCtas)) * (KP * 8);
+    return a + (uint32_t)(col - (int)((long long)n * own / kLcCtas)) * (KP * 8);
+  };
+  for (int p = tid; p < min(nz, zcap); p += kLcThreads) {
+    ps[p] = p_row(__ldg(ci + p0 + p));
     as[p] = __ldg(av + p0 + p);
   }
   for (int i = tid; i <= r1 - r0; i += kLcThreads) rs[i] = __ldg(rp + r0 + i) - p0;
@@ -368,13 +372,31 @@ k_loop_cluster(int n, const int* __restrict__ rp, const int* __restrict__ ci, co
       if (e < tot) {
         const int i = e / KP, pe = rs[i + 1];
         constexpr int kB = 8;  // entries of a row in flight together
-        for (int p = rs[i]; p < pe; p += kB) {
-          double x[kB];
+        if (pe <= zcap) {
+          for (int p = rs[i]; p < pe; p += kB) {
+            double x[kB];
 #pragma unroll
-          for (int b = 0; b < kB; ++b) x[b] = p + b < pe ? ld_cluster(ps[p + b] + m * 8) : 0.0;
+            for (int b = 0; b < kB; ++b) x[b] = p + b < pe ? ld_cluster(ps[p + b] + m * 8) : 0.0;
 #pragma unroll
-          for (int b = 0; b < kB; ++b)
-            if (p + b < pe) acc = fma(as[p + b], x[b], acc);
+            for (int b = 0; b < kB; ++b)
+              if (p + b < pe) acc = fma(as[p + b], x[b], acc);
+          }
+        } else {
+          for (int p = rs[i]; p < pe; p += kB) {
+            double x[kB], a[kB];
+            int c[kB];
+#pragma unroll
+            for (int b = 0; b < kB; ++b) {
+              const int q = p0 + min(p + b, pe - 1);
+              c[b] = __ldg(ci + q);
+              a[b] = __ldg(av + q);
+            }
+#pragma unroll
+            for (int b = 0; b < kB; ++b) x[b] = ld_cluster(p_row(c[b]) + m * 8);
+#pragma unroll
+            for (int b = 0; b < kB; ++b)
+              if (p + b < pe) acc = fma(a[b], x[b], acc);
+          }
         }
         pm = P[e];
         Q[e] = acc;
@@ -626,13 +648,13 @@ __global__ void k_lc_slice(int n, const int* __restrict__ rp, int* out) {
   if (threadIdx.x == 0) *out = v;
 }
 
-size_t lc_smem(int kp, int n, int slice) {
+size_t lc_smem(int kp, int n, int zcap) {
   const int rows = (n + kLcCtas - 1) / kLcCtas;
-  return 6 * (size_t)((rows * kp + 1) & ~1) * sizeof(double) + (size_t)slice * 12 + (size_t)(rows + 1) * 4;
+  return 6 * (size_t)((rows * kp + 1) & ~1) * sizeof(double) + (size_t)zcap * 12 + (size_t)(rows + 1) * 4;
 }
 
 using LcKernel = void (*)(int, const int*, const int*, const double*, double*, double*, double*, double*, const double*,
-                          double*, SolveState*, int, cudaGraphConditionalHandle, int);
+                          double*, SolveState*, int, int, cudaGraphConditionalHandle, int);
 
 LcKernel lc_kernel(int kp) {
   switch (kp) {
@@ -643,11 +665,11 @@ LcKernel lc_kernel(int kp) {
   }
 }
 
-cudaLaunchConfig_t lc_config(int kp, int n, int slice, cudaStream_t s, cudaLaunchAttribute* at) {
+cudaLaunchConfig_t lc_config(int kp, int n, int zcap, cudaStream_t s, cudaLaunchAttribute* at) {
   cudaLaunchConfig_t c = {};
   c.gridDim = dim3(kLcCtas);
   c.blockDim = dim3(kLcThreads);
-  c.dynamicSmemBytes = lc_smem(kp, n, slice);
+  c.dynamicSmemBytes = lc_smem(kp, n, zcap);
   c.stream = s;
   at->id = cudaLaunchAttributeClusterDimension;
   at->val.clusterDim.x = kLcCtas;
@@ -674,28 +696,31 @@ bool loop_cluster_fits(int kp, int n, long long nnz) {
 
 void loop_cluster_slice(cudaStream_t s, int n, const int* rp, int* out) { k_lc_slice<<<1, 32, 0, s>>>(n, rp, out); }
 
-bool loop_cluster_ready(int kp, int n, int slice) {
+int loop_cluster_ready(int kp, int n, int slice) {
   constexpr size_t kSmem = 227 * 1024;
   const LcKernel k = lc_kernel(kp);
   cudaFuncAttributes fa;
   cudaLaunchAttribute at;
-  const cudaLaunchConfig_t c = lc_config(kp, n, slice, nullptr, &at);
-  int clusters = 0;
-  const bool ok = cudaFuncGetAttributes(&fa, k) == cudaSuccess && c.dynamicSmemBytes + fa.sharedSizeBytes <= kSmem &&
-                  cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
-                  cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)(kSmem - fa.sharedSizeBytes)) == cudaSuccess &&
-                  cudaOccupancyMaxActiveClusters(&clusters, k, &c) == cudaSuccess;
-  if (!ok) cudaGetLastError();
-  return ok && clusters > 0;
+  int clusters = 0, zcap = -1;
+  bool ok = cudaFuncGetAttributes(&fa, k) == cudaSuccess && lc_smem(kp, n, 0) + fa.sharedSizeBytes <= kSmem;
+  if (ok) {
+    zcap = (int)std::min((size_t)slice, (kSmem - fa.sharedSizeBytes - lc_smem(kp, n, 0)) / 12);
+    const cudaLaunchConfig_t c = lc_config(kp, n, zcap, nullptr, &at);
+    ok = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+         cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kSmem - fa.sharedSizeBytes)) ==
+             cudaSuccess &&
+         cudaOccupancyMaxActiveClusters(&clusters, k, &c) == cudaSuccess;
+  }
+  cudaGetLastError();  // a refusal here only means the launches of the row kernels
+  return ok && clusters > 0 && 2 * (long long)zcap >= slice ? zcap : -1;
 }
 
 void launch_loop_cluster(cudaStream_t s, int kp, const LoopArgs& a, int iters, cudaGraphConditionalHandle cond,
                          int use_cond) {
   cudaLaunchAttribute at;
-  const cudaLaunchConfig_t c = lc_config(kp, a.n, a.slice, s, &at);
+  const cudaLaunchConfig_t c = lc_config(kp, a.n, a.zcap, s, &at);
   cudaLaunchKernelEx(&c, lc_kernel(kp), a.n, a.rp, a.ci, a.av, a.X, a.R, a.W, a.P, a.wdiag, a.Sigma,
-                     a.st, iters, cond, use_cond);
+                     a.st, a.zcap, iters, cond, use_cond);
 }
 
 }  // namespace mbpcg
