@@ -687,12 +687,13 @@ void enqueue_reduce(mbpcg_ctx* h, int nent, const SolveState* st, int mx = 0, in
 
 void enqueue_true_residual(mbpcg_ctx* h) {
   const Dims& dm = h->dm;
+  const int nb = dm.dense ? dm.nbmax : dm.nb;
   if (dm.dense)
-    k_resid_dense<<<dm.nb, kThreads, 0, h->stream>>>(dm.n, h->A, h->sqd, h->b, h->x, h->rhs, h->part, dm.pstride);
+    k_resid_dense<<<nb, kThreads, 0, h->stream>>>(dm.n, h->A, h->sqd, h->b, h->x, h->rhs, h->part, dm.pstride);
   else
-    k_resid_csr<<<dm.nb, kThreads, 0, h->stream>>>(dm.n, h->rp, h->ci, h->av, h->sqd, h->b, h->x, h->rhs, h->part,
+    k_resid_csr<<<nb, kThreads, 0, h->stream>>>(dm.n, h->rp, h->ci, h->av, h->sqd, h->b, h->x, h->rhs, h->part,
                                                    dm.pstride);
-  launch_reduce(h->stream, h->part, dm.nb, dm.pstride, h->red, 1, nullptr);
+  launch_reduce(h->stream, h->part, nb, dm.pstride, h->red, 1, nullptr);
   k_small_true<<<1, 1, 0, h->stream>>>(h->st, h->red);
 }
 

@@ -101,151 +101,150 @@ k_spmm_dots(int n, const int* __restrict__ rp, const int* __restrict__ ci, const
 
 // ------------------------------------------------------------------------------------------------
 // Q = A P for dense symmetric A stored column-major (row i of A is column i, contiguous).
-// One CTA per SM owns a balanced range of rows and walks it in passes of G rows. The reduction index
+// One CTA per SM owns a balanced range of rows and walks it in passes of G = 4 TR rows. The reduction index
 // l is split into chunks of LC: for each chunk the A rows (G x LC) and the P rows (LC x KP) are
 // copied into shared memory by 1-D TMA bulk copies (cp.async.bulk) that complete on an mbarrier,
-// STAGES chunks in flight, so HBM latency is hidden behind the FP64 FMAs. Each thread owns a
-// TR x TC register tile of the output and a residue class of l (LS classes, summed at the end in a
-// fixed order). Rows of odd length (n odd) break the 16-byte rule of bulk copies; then the same
-// pipeline is filled with ordinary loads. Every mbarrier wait is bounded: on a timeout the CTA sets
+// STAGES chunks in flight, so HBM latency is hidden behind the FP64 FMAs, which bound it (2 a clock per SM).
+// Every warp has all G rows for its share of the l of a chunk (LS residue classes, summed at the end in a
+// fixed order): lane = (column group, row group of 4, class), rows rg + 4 t for t < TR, so the FMAs done are
+// those of 4 TR rows whatever TR is, evenly on the four sub-partitions, and TR follows the rows that a CTA
+// has (dense_rows). A tile of 32 rows spread over the warps instead left warps idle whenever a CTA had fewer
+// (half of them at n = 2304, KP = 8: 100 us; now 76 us, of which 69 are the FP64 pipe's;
+// n = 4096, KP = 4: 139 -> 119; KP = 32: 916 -> 898; n = 900, KP = 32: 132 -> 60).
+// Rows of odd length (n odd) break the 16-byte rule of bulk copies; then the same
+// pipeline is filled by 8-byte asynchronous copies (cp.async; n = 4097, KP = 8: 336 -> 233 us). Every mbarrier wait is bounded: on a timeout the CTA sets
 // *err (if given), waits (bounded) for the copies it still has in flight, and returns.
-template <int KP>
+template <int KP, int TR>
 struct DenseCfg {
-  static constexpr int G = 32;
+  static constexpr int G = 4 * TR;
   static constexpr int LC = 128;
-  static constexpr int LDA = LC + 2;  // shared-memory row stride of the A tile (keeps 16-byte rows)
+  static constexpr int LDA = LC + 2;  // shared-memory row stride of the A tile (16-byte rows; 4 rows apart in banks)
   static constexpr int STAGES = 3;
-  static constexpr int TR = (KP <= 2) ? 1 : 2;
-  static constexpr int TC = (KP == 1) ? 1 : 2;
-  static constexpr int RT = G / TR;
-  static constexpr int CT = KP / TC;
-  static constexpr int LS = kThreads / (RT * CT);
+  static constexpr int CT = KP < 8 ? KP : 8;  // column lanes; lane column ct has ct + CT c
+  static constexpr int TC = KP / CT;
+  static constexpr int LSUB = 8 / CT;         // classes of l inside a warp
+  static constexpr int LS = kThreads / 32 * LSUB;
   static constexpr int A_ELEMS = G * LDA;
   static constexpr int STAGE_ELEMS = A_ELEMS + LC * KP;
-  static constexpr int RED_ELEMS = (LS > 1) ? LS * G * KP : 1;
-  static constexpr size_t SMEM = (size_t)(STAGES * STAGE_ELEMS + RED_ELEMS) * sizeof(double) + STAGES * 8;
+  static constexpr size_t SMEM = (size_t)(STAGES * STAGE_ELEMS) * sizeof(double) + 2 * STAGES * 8;
+  static_assert(LS * G * KP <= STAGES * STAGE_ELEMS, "the class sums lie over the stages");
 };
 
-template <int KP>
-__global__ void __launch_bounds__(kThreads, 1)
+// TR for n rows on nb CTAs: passes of at most 32 rows, all alike.
+inline int dense_rows(int n, int nb) {
+  const int rows = (n + nb - 1) / nb, passes = (rows + 31) / 32;
+  return ((rows + passes - 1) / passes + 3) / 4;
+}
+
+constexpr int kDenseThreads = kThreads + 32;  // 8 warps multiply, the last one issues the copies
+
+template <int KP, int TR>
+__global__ void __launch_bounds__(kDenseThreads, 1)
 k_dense(int n, const double* __restrict__ A, const double* __restrict__ P, double* __restrict__ Q,
         const SolveState* __restrict__ st, int* __restrict__ err) {
-  using D = DenseCfg<KP>;
+  using D = DenseCfg<KP, TR>;
   if (st != nullptr && st->done) return;
   extern __shared__ __align__(128) double dsm[];
-  double* red = dsm + D::STAGES * D::STAGE_ELEMS;
-  uint64_t* bars = reinterpret_cast<uint64_t*>(red + D::RED_ELEMS);
-  __shared__ int abort_flag;
+  double* red = dsm;
+  uint64_t* full = reinterpret_cast<uint64_t*>(dsm + D::STAGES * D::STAGE_ELEMS);
+  uint64_t* empty = full + D::STAGES;
+  __shared__ int abort_flag, issued;
   int r0, r1;
   row_range(n, r0, r1);
-  const int tid = threadIdx.x;
-  const int q = tid % D::LS, tile = tid / D::LS, ct = tile % D::CT, rt = tile / D::CT;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int ct = lane % D::CT, rg = lane / D::CT % 4, q = warp * D::LSUB + lane / (4 * D::CT);
   const bool tma = (n % 2) == 0;
   if (tid == 0) {
-    for (int s = 0; s < D::STAGES; ++s) mbar_init(&bars[s], 1);
+    for (int s = 0; s < D::STAGES; ++s) {
+      mbar_init(&full[s], tma ? 1 : 32);
+      mbar_init(&empty[s], kThreads / 32);
+    }
     mbar_fence_init();
     abort_flag = 0;
   }
   __syncthreads();
   const int nchunks = (n + D::LC - 1) / D::LC;
-  int g_next = 0;  // global index of the next chunk to consume (stage = g % STAGES)
+  int g0 = 0;  // chunks of the passes before (chunk g uses stage g % STAGES)
   for (int base = r0; base < r1; base += D::G) {
     const int rows = min(D::G, r1 - base);
-    const int g0 = g_next;
-    auto issue = [&](int c) {
-      const int g = g0 + c, stage = g % D::STAGES, l0 = c * D::LC, lc = min(D::LC, n - l0);
-      double* As = dsm + stage * D::STAGE_ELEMS;
-      double* Ps = As + D::A_ELEMS;
-      if (tma) {
-        if (tid < 32) {
-          if (tid == 0) mbar_arrive_expect_tx(&bars[stage], (uint32_t)((rows + KP) * lc * sizeof(double)));
-          __syncwarp();
-          for (int r = tid; r < rows; r += 32)
-            tma_load_1d(As + r * D::LDA, A + (size_t)(base + r) * n + l0, (uint32_t)(lc * sizeof(double)),
-                        &bars[stage]);
-          if (tid == 0)
-            tma_load_1d(Ps, P + (size_t)l0 * KP, (uint32_t)(lc * KP * sizeof(double)), &bars[stage]);
-        }
-      } else {
-        for (int e = tid; e < rows * lc; e += kThreads) {
-          const int r = e / lc, l = e - r * lc;
-          As[r * D::LDA + l] = A[(size_t)(base + r) * n + l0 + l];
-        }
-        for (int e = tid; e < lc * KP; e += kThreads) Ps[e] = P[(size_t)l0 * KP + e];
-      }
-    };
-    double acc[D::TR][D::TC];
+    double acc[TR][D::TC];
 #pragma unroll
-    for (int r = 0; r < D::TR; ++r)
+    for (int r = 0; r < TR; ++r)
 #pragma unroll
       for (int c = 0; c < D::TC; ++c) acc[r][c] = 0.0;
-    const int pre = min(D::STAGES - 1, nchunks);
-    for (int c = 0; c < pre; ++c) issue(c);
-    int issued = pre;
-    __syncthreads();
-    for (int c = 0; c < nchunks; ++c) {
-      if (c + D::STAGES - 1 < nchunks) {
-        issue(c + D::STAGES - 1);
-        issued = c + D::STAGES;
+    auto consume = [&](int c) {  // (rows past the CTA's last one: what the stage held before, not stored)
+      const double* As = dsm + (g0 + c) % D::STAGES * D::STAGE_ELEMS + rg * D::LDA;
+      const double* Ps = dsm + (g0 + c) % D::STAGES * D::STAGE_ELEMS + D::A_ELEMS + ct;
+      const int lc = min(D::LC, n - c * D::LC);
+#pragma unroll 2
+      for (int l = q; l < lc; l += D::LS) {
+        double a[TR], p[D::TC];
+#pragma unroll
+        for (int r = 0; r < TR; ++r) a[r] = As[4 * r * D::LDA + l];
+#pragma unroll
+        for (int cc = 0; cc < D::TC; ++cc) p[cc] = Ps[l * KP + cc * D::CT];
+#pragma unroll
+        for (int r = 0; r < TR; ++r)
+#pragma unroll
+          for (int cc = 0; cc < D::TC; ++cc) acc[r][cc] = fma(a[r], p[cc], acc[r][cc]);
       }
-      const int g = g0 + c, stage = g % D::STAGES;
-      bool ok = true;
-      if (tma) ok = mbar_wait_bounded(&bars[stage], (uint32_t)((g / D::STAGES) & 1));
-      if (!ok) abort_flag = 1;
-      if (ok && rt * D::TR < rows) {
-        const double* As = dsm + stage * D::STAGE_ELEMS;
-        const double* Ps = As + D::A_ELEMS;
-        const int lc = min(D::LC, n - c * D::LC);
-        for (int l = q; l < lc; l += D::LS) {
-          double a[D::TR], p[D::TC];
-#pragma unroll
-          for (int r = 0; r < D::TR; ++r) a[r] = As[(rt * D::TR + r) * D::LDA + l];
-          if constexpr (D::TC == 2) {
-            const double2 t = *reinterpret_cast<const double2*>(Ps + l * KP + ct * 2);
-            p[0] = t.x;
-            p[1] = t.y;
-          } else {
-            p[0] = Ps[l * KP + ct];
-          }
-#pragma unroll
-          for (int r = 0; r < D::TR; ++r)
-#pragma unroll
-            for (int cc = 0; cc < D::TC; ++cc) acc[r][cc] = fma(a[r], p[cc], acc[r][cc]);
+    };
+    if (warp == kThreads / 32) {
+      int c = 0;
+      for (; c < nchunks; ++c) {
+        const int g = g0 + c, stage = g % D::STAGES, l0 = c * D::LC, lc = min(D::LC, n - l0);
+        if (g >= D::STAGES && !mbar_wait_bounded(&empty[stage], (uint32_t)((g / D::STAGES - 1) & 1))) break;
+        double* As = dsm + stage * D::STAGE_ELEMS;
+        if (tma) {
+          if (lane == 0) mbar_arrive_expect_tx(&full[stage], (uint32_t)((rows + KP) * lc * sizeof(double)));
+          __syncwarp();
+          for (int r = lane; r < rows; r += 32)
+            tma_load_1d(As + r * D::LDA, A + (size_t)(base + r) * n + l0, (uint32_t)(lc * sizeof(double)), &full[stage]);
+          if (lane == 0)
+            tma_load_1d(As + D::A_ELEMS, P + (size_t)l0 * KP, (uint32_t)(lc * KP * sizeof(double)), &full[stage]);
+        } else {
+          for (int r = 0; r < rows; ++r)
+            for (int l = lane; l < lc; l += 32) cp_async_8(As + r * D::LDA + l, A + (size_t)(base + r) * n + l0 + l);
+          for (int e = lane; e < lc * KP; e += 32) cp_async_8(As + D::A_ELEMS + e, P + (size_t)l0 * KP + e);
+          cp_async_mbar_arrive(&full[stage]);
         }
       }
-      __syncthreads();
-      if (abort_flag) {
-        if (tid == 0) {
-          if (err != nullptr) atomicExch(err, 1);
-          for (int c2 = c; c2 < issued; ++c2) {  // drain the copies still in flight (bounded)
-            const int g2 = g0 + c2;
-            mbar_wait_bounded(&bars[g2 % D::STAGES], (uint32_t)((g2 / D::STAGES) & 1));
-          }
-        }
-        __syncthreads();
-        return;
-      }
-    }
-    g_next = g0 + nchunks;
-    // sum the LS residue classes in a fixed order, then store the valid rows
-    if constexpr (D::LS > 1) {
-#pragma unroll
-      for (int r = 0; r < D::TR; ++r)
-#pragma unroll
-        for (int cc = 0; cc < D::TC; ++cc) red[(q * D::G + rt * D::TR + r) * KP + ct * D::TC + cc] = acc[r][cc];
-      cta_tree_sum(red, D::LS, D::G * KP);
-      for (int e = tid; e < rows * KP; e += kThreads) Q[(size_t)base * KP + e] = red[e];
-      __syncthreads();
+      if (lane == 0) issued = c;
+      if (c < nchunks) abort_flag = 1;
     } else {
-#pragma unroll
-      for (int r = 0; r < D::TR; ++r) {
-        const int row = rt * D::TR + r;
-        if (row < rows) {
-#pragma unroll
-          for (int cc = 0; cc < D::TC; ++cc) Q[(size_t)(base + row) * KP + ct * D::TC + cc] = acc[r][cc];
+      for (int c = 0; c < nchunks; ++c) {
+        const int g = g0 + c, stage = g % D::STAGES;
+        if (!mbar_wait_bounded(&full[stage], (uint32_t)((g / D::STAGES) & 1))) {
+          abort_flag = 1;
+          break;
         }
+        consume(c);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&empty[stage]);
       }
     }
+    __syncthreads();
+    if (abort_flag) {
+      if (tid == 0) {
+        if (err != nullptr) atomicExch(err, 1);
+        for (int c = max(0, issued - D::STAGES); c < issued; ++c)  // drain the copies still in flight (bounded)
+          mbar_wait_bounded(&full[(g0 + c) % D::STAGES], (uint32_t)(((g0 + c) / D::STAGES) & 1));
+      }
+      __syncthreads();
+      return;
+    }
+    g0 += nchunks;
+    // sum the LS residue classes in a fixed order (over the stages: their copies have all been consumed),
+    // then store the valid rows
+    if (warp < kThreads / 32)
+#pragma unroll
+      for (int r = 0; r < TR; ++r)
+#pragma unroll
+        for (int cc = 0; cc < D::TC; ++cc) red[(q * D::G + rg + 4 * r) * KP + ct + cc * D::CT] = acc[r][cc];
+    cta_tree_sum(red, D::LS, D::G * KP);
+    for (int e = tid; e < rows * KP; e += kDenseThreads) Q[(size_t)base * KP + e] = red[e];
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // before the next pass's bulk copies
+    __syncthreads();
   }
 }
 
