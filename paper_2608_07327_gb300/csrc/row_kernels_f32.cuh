@@ -81,6 +81,48 @@ __device__ __forceinline__ void dot2_add(float& s, float& c, float x, float y) {
   c = __fadd_rn(c, __fadd_rn(se, pe));
 }
 
+// Two FP32 numbers in one register pair, for the packed FP32 instructions: the same roundings as the scalar
+// ones with half the instructions to issue (27-point 96^3, KP = 16: the block update 169 -> 154 us, the Gram of
+// the product 64.6 -> 63.7).
+struct f32x2 {
+  unsigned long long v;
+};
+__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void unpack2(f32x2 a, float& lo, float& hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(a.v));
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+  return r;
+}
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) { return fma2(b, pack2(-1.f, -1.f), a); }
+
+// dot2_add on two independent sums, the same bits; ny = -y.
+__device__ __forceinline__ void dot2_add2(f32x2& s, f32x2& c, f32x2 x, f32x2 y, f32x2 ny) {
+  const f32x2 np = mul2(x, ny);  // -p
+  const f32x2 pe = fma2(x, y, np);
+  const f32x2 t = sub2(s, np);
+  const f32x2 z = sub2(t, s);
+  const f32x2 se = sub2(sub2(s, sub2(t, z)), add2(np, z));
+  s = t;
+  c = add2(c, add2(se, pe));
+}
+
 // Upper triangle of X^T Y over a tile of FP32 rows in shared memory (row stride KP), with Dot2
 // accumulators; same thread layout as GramTile (2 x 2 blocks, row classes), FP64 partials.
 template <int KP>
@@ -91,7 +133,7 @@ struct GramTileF {
   static constexpr int RED = RS * NBLK * 4;  // doubles of shared scratch for finish()
   int bl, bj, blk, split;
   bool active;
-  float s00, s01, s10, s11, c00, c01, c10, c11;
+  f32x2 s0, s1, c0, c1;  // entries (2 bl, 2 bj), (2 bl, 2 bj + 1) in 0, those of 2 bl + 1 in 1
 
   __device__ __forceinline__ void init(int tid) {
     active = tid < NBLK * RS;
@@ -100,20 +142,22 @@ struct GramTileF {
     bj = 0;
     while ((bj + 1) * (bj + 2) / 2 <= blk) ++bj;
     bl = blk - bj * (bj + 1) / 2;
-    s00 = s01 = s10 = s11 = c00 = c01 = c10 = c11 = 0.f;
+    s0 = s1 = c0 = c1 = f32x2{0ull};
   }
   __device__ __forceinline__ void accumulate(const float* Xs, const float* Ys, int nrows) {
     if (!active) return;
     if constexpr (KP == 1) {
-      for (int r = split; r < nrows; r += RS) dot2_add(s00, c00, Xs[r], Ys[r]);
+      for (int r = split; r < nrows; r += RS) {
+        const float y = Ys[r];
+        dot2_add2(s0, c0, pack2(Xs[r], 0.f), pack2(y, 0.f), pack2(-y, 0.f));
+      }
     } else {
       for (int r = split; r < nrows; r += RS) {
         const float2 x = *reinterpret_cast<const float2*>(Xs + r * KP + 2 * bl);
         const float2 y = *reinterpret_cast<const float2*>(Ys + r * KP + 2 * bj);
-        dot2_add(s00, c00, x.x, y.x);
-        dot2_add(s01, c01, x.x, y.y);
-        dot2_add(s10, c10, x.y, y.x);
-        dot2_add(s11, c11, x.y, y.y);
+        const f32x2 yy = pack2(y.x, y.y), ny = pack2(-y.x, -y.y);
+        dot2_add2(s0, c0, pack2(x.x, x.x), yy, ny);
+        dot2_add2(s1, c1, pack2(x.y, x.y), yy, ny);
       }
     }
   }
@@ -121,10 +165,13 @@ struct GramTileF {
     __syncthreads();
     if (active) {
       const int o = (split * NBLK + blk) * 4;
-      red[o] = (double)s00 + (double)c00;
-      red[o + 1] = (double)s01 + (double)c01;
-      red[o + 2] = (double)s10 + (double)c10;
-      red[o + 3] = (double)s11 + (double)c11;
+      float s[4], c[4];
+      unpack2(s0, s[0], s[1]);
+      unpack2(s1, s[2], s[3]);
+      unpack2(c0, c[0], c[1]);
+      unpack2(c1, c[2], c[3]);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) red[o + e] = (double)s[e] + (double)c[e];
     }
     cta_tree_sum(red, RS, NBLK * 4);
     for (int e = threadIdx.x; e < KP * (KP + 1) / 2; e += blockDim.x) {
