@@ -24,15 +24,23 @@ k_spmm(int n, const int* __restrict__ rp, const int* __restrict__ ci, const doub
   using C = Cfg<KP>;
   using G = GramTile<KP>;
   if (st != nullptr && st->done) return;
-  __shared__ __align__(16) double Xs[GRAM ? C::ROWS * KP : 2];
-  __shared__ __align__(16) double Ys[GRAM ? C::ROWS * KP : 2];
-  __shared__ __align__(16) double red[GRAM ? G::RED : 2];
+  // A thread that has whole rows (KP <= 4) sums the Gram's terms of its rows in registers: KP (KP + 1) / 2 FMAs
+  // a row and no barrier (diffusion 128^3, KP = 4: 148 us with the Gram against 167 by tiles; 129 us of
+  // the FP64 pipe; KP = 2 89 -> 77, KP = 1 59 -> 50; Poisson 160^2, KP = 4 11.5 -> 9.0).
+  constexpr bool kRegs = C::TPR == 1;
+  __shared__ __align__(16) double Xs[GRAM && !kRegs ? C::ROWS * KP : 2];
+  __shared__ __align__(16) double Ys[GRAM && !kRegs ? C::ROWS * KP : 2];
+  __shared__ __align__(16) double red[GRAM ? (kRegs ? C::NPACK * kThreads : G::RED) : 2];
   int r0, r1;
   row_range(n, r0, r1);
   const int tid = threadIdx.x;
   const int rl = tid / C::TPR, j0 = (tid % C::TPR) * C::CPT;
   G g;
-  if constexpr (GRAM) g.init(tid);
+  double gs[kRegs ? C::NPACK : 1];
+  if constexpr (GRAM && !kRegs) g.init(tid);
+  if constexpr (GRAM && kRegs)
+#pragma unroll
+    for (int e = 0; e < C::NPACK; ++e) gs[e] = 0.0;
   for (int base = r0; base < r1; base += C::ROWS) {
     const int i = base + rl;
     double acc[C::CPT], pv[C::CPT];
@@ -51,8 +59,13 @@ k_spmm(int n, const int* __restrict__ rp, const int* __restrict__ ci, const doub
       }
       stv<C::CPT>(Q + (size_t)i * KP + j0, acc);
       if constexpr (GRAM) ldv<C::CPT>(P + (size_t)i * KP + j0, pv);
+      if constexpr (GRAM && kRegs)
+#pragma unroll
+        for (int m = 0; m < KP; ++m)
+#pragma unroll
+          for (int l = 0; l <= m; ++l) gs[m * (m + 1) / 2 + l] = fma(pv[l], acc[m], gs[m * (m + 1) / 2 + l]);
     }
-    if constexpr (GRAM) {
+    if constexpr (GRAM && !kRegs) {
 #pragma unroll
       for (int c = 0; c < C::CPT; ++c) {
         Xs[rl * KP + j0 + c] = pv[c];
@@ -63,7 +76,14 @@ k_spmm(int n, const int* __restrict__ rp, const int* __restrict__ ci, const doub
       __syncthreads();
     }
   }
-  if constexpr (GRAM) g.finish(red, part + (size_t)blockIdx.x * pstride);
+  if constexpr (GRAM && kRegs) {
+#pragma unroll
+    for (int e = 0; e < C::NPACK; ++e) red[tid * C::NPACK + e] = gs[e];
+    cta_tree_sum(red, min(kThreads, r1 - r0), C::NPACK);
+    if (tid < C::NPACK) part[(size_t)blockIdx.x * pstride + tid] = r1 > r0 ? red[tid] : 0.0;
+  } else if constexpr (GRAM) {
+    g.finish(red, part + (size_t)blockIdx.x * pstride);
+  }
 }
 
 // The same for one column, w = A r, with the CTA partials of (r, r), (w, r) and ||D r||^2 (wdiag = D^2 or
@@ -406,14 +426,17 @@ k_axpy(int n, const double* __restrict__ P, const double* __restrict__ Q, const 
        double* __restrict__ part, int pstride, const SolveState* __restrict__ st) {
   using C = Cfg<KP>;
   using G = GramTile<KP>;
-  constexpr int RED = (G::RED > C::ROWS * KP) ? G::RED : C::ROWS * KP;
+  constexpr bool kRegs = C::TPR == 1;
+  constexpr int NS = C::NPACK + (RFREE ? C::NPACK : KP);  // sums of a thread that has whole rows
+  constexpr int RED = kRegs ? NS * kThreads : (G::RED > C::ROWS * KP) ? G::RED : C::ROWS * KP;
+  constexpr int TILE = kRegs ? 2 : C::ROWS * KP;
   if (st->done) return;
   __shared__ __align__(16) double Ts[KP * KP];
   __shared__ __align__(16) double Xis[KP * KP];
-  __shared__ __align__(16) double Ps[C::ROWS * KP];
-  __shared__ __align__(16) double Qs[C::ROWS * KP];
-  __shared__ __align__(16) double Vs[C::ROWS * KP];
-  __shared__ __align__(16) double Vws[RFREE ? C::ROWS * KP : 2];
+  __shared__ __align__(16) double Ps[TILE];
+  __shared__ __align__(16) double Qs[TILE];
+  __shared__ __align__(16) double Vs[TILE];
+  __shared__ __align__(16) double Vws[RFREE ? TILE : 2];
   __shared__ __align__(16) double red[RED];
   const bool wgram = RFREE && wdiag != nullptr;
   const int tid = threadIdx.x, rl = tid / C::TPR, j0 = (tid % C::TPR) * C::CPT;
@@ -424,6 +447,60 @@ k_axpy(int n, const double* __restrict__ P, const double* __restrict__ Q, const 
   }
   int r0, r1;
   row_range(n, r0, r1);
+  // whole rows: Gram terms and norms in registers, as in k_spmm (Poisson 160^2, KP = 4: 15.8 -> 14.1 us; 36^3,
+  // KP = 2, implicit residual 13.8 -> 8.1; diffusion 128^3, KP = 2 96 -> 86, KP = 1 29.6 -> 30.5)
+  if constexpr (kRegs) {
+    __syncthreads();
+    double sum[NS];
+#pragma unroll
+    for (int e = 0; e < NS; ++e) sum[e] = 0.0;
+    for (int i = r0 + tid; i < r1; i += kThreads) {
+      double p[KP], q[KP], x[KP], r[KP], v[KP];
+      ldv<KP>(P + (size_t)i * KP, p);
+      ldv<KP>(Q + (size_t)i * KP, q);
+      ldv_plain<KP>(Xt + (size_t)i * KP, x);
+      if constexpr (!RFREE) ldv_plain<KP>(R + (size_t)i * KP, r);
+      ldv<KP>(W + (size_t)i * KP, v);
+#pragma unroll
+      for (int l = 0; l < KP; ++l)
+#pragma unroll
+        for (int c = 0; c < KP; ++c) {
+          const double tl = Ts[l * KP + c];
+          x[c] = fma(p[l], tl, x[c]);
+          if constexpr (!RFREE) r[c] = fma(-q[l], tl, r[c]);
+          v[c] = fma(-q[l], Xis[l * KP + c], v[c]);
+        }
+      stv<KP>(Xt + (size_t)i * KP, x);
+      stv<KP>(V + (size_t)i * KP, v);
+#pragma unroll
+      for (int m = 0; m < KP; ++m)
+#pragma unroll
+        for (int l = 0; l <= m; ++l) sum[m * (m + 1) / 2 + l] = fma(v[l], v[m], sum[m * (m + 1) / 2 + l]);
+      if constexpr (!RFREE) {
+        stv<KP>(R + (size_t)i * KP, r);
+        const double w2 = wdiag != nullptr ? __ldg(wdiag + i) : 1.0;
+#pragma unroll
+        for (int c = 0; c < KP; ++c)
+          sum[C::NPACK + c] = fma(wdiag != nullptr ? r[c] * w2 : r[c], r[c], sum[C::NPACK + c]);
+      } else if (wgram) {
+        const double w2 = __ldg(wdiag + i);
+#pragma unroll
+        for (int m = 0; m < KP; ++m) {
+          const double wv = w2 * v[m];
+#pragma unroll
+          for (int l = 0; l <= m; ++l)
+            sum[C::NPACK + m * (m + 1) / 2 + l] = fma(v[l], wv, sum[C::NPACK + m * (m + 1) / 2 + l]);
+        }
+      }
+    }
+#pragma unroll
+    for (int e = 0; e < NS; ++e) red[tid * NS + e] = sum[e];
+    cta_tree_sum(red, min(kThreads, r1 - r0), NS);
+    double* out = part + (size_t)blockIdx.x * pstride;
+    if (tid < (RFREE && !wgram ? C::NPACK : NS))  // V^T V, then nu; RFREE: V^T D^2 V after nu's place
+      out[tid + (RFREE && tid >= C::NPACK ? KP : 0)] = r1 > r0 ? red[tid] : 0.0;
+    return;
+  }
   G g, g2;
   g.init(tid);
   if (wgram) g2.init(tid);
@@ -830,43 +907,65 @@ __global__ void k_gen_u(int n, int s, unsigned long long seed, double* __restric
   }
 }
 
-// Column-major n x s (leading dimension n) <-> row-major n x KP with zero padding, by tiles of
+// Column-major n x s (leading dimension n) <-> row-major n x KP with zero padding. From KP = 8 by tiles of
 // kTrRows rows turned in shared memory so that both sides move whole 128-byte lines: 27-point 96^3, KP = 16,
-// s = 16: 152 -> 37 us (a thread per value, one side strided by n).
+// s = 16: 152 -> 37 us. Below, a thread per value: its strided side still fills 32-byte sectors together with
+// its neighbours' (diffusion 128^3 out of KP = 4, 2, 1: 23, 13, 9 us against 39, 33, 28 by tiles).
 constexpr int kTrRows = 64;
+constexpr int kTrMinKP = 8;
 template <int KP>
 struct TransposeTile {
   static constexpr int LD = kTrRows + 1;
   double v[KP * LD];  // v[j * LD + r]
 };
 template <int KP>
-__global__ void __launch_bounds__(kThreads) k_from_colmajor(int n, int s, const double* __restrict__ src, double* __restrict__ dst) {
-  using T = TransposeTile<KP>;
-  __shared__ T t;
-  for (int r0 = blockIdx.x * kTrRows; r0 < n; r0 += gridDim.x * kTrRows) {
-    const int rows = min(kTrRows, n - r0);
-    for (int q = threadIdx.x; q < KP * kTrRows; q += kThreads) {
-      const int j = q / kTrRows, r = q % kTrRows;
-      t.v[j * T::LD + r] = (j < s && r < rows) ? src[(size_t)j * n + r0 + r] : 0.0;
+__global__ void __launch_bounds__(kThreads)
+k_from_colmajor(int n, int s, const double* __restrict__ src, double* __restrict__ dst) {
+  if constexpr (KP < kTrMinKP) {
+    const size_t total = (size_t)n * KP;
+    for (size_t q = blockIdx.x * (size_t)kThreads + threadIdx.x; q < total; q += (size_t)gridDim.x * kThreads) {
+      const int j = (int)(q % KP);
+      dst[q] = j < s ? src[(size_t)j * n + q / KP] : 0.0;
     }
-    __syncthreads();
-    for (int q = threadIdx.x; q < rows * KP; q += kThreads) dst[(size_t)r0 * KP + q] = t.v[(q % KP) * T::LD + q / KP];
-    __syncthreads();
+  } else {
+    using T = TransposeTile<KP>;
+    __shared__ T t;
+    for (int r0 = blockIdx.x * kTrRows; r0 < n; r0 += gridDim.x * kTrRows) {
+      const int rows = min(kTrRows, n - r0);
+      for (int q = threadIdx.x; q < KP * kTrRows; q += kThreads) {
+        const int j = q / kTrRows, r = q % kTrRows;
+        t.v[j * T::LD + r] = (j < s && r < rows) ? src[(size_t)j * n + r0 + r] : 0.0;
+      }
+      __syncthreads();
+      for (int q = threadIdx.x; q < rows * KP; q += kThreads)
+        dst[(size_t)r0 * KP + q] = t.v[(q % KP) * T::LD + q / KP];
+      __syncthreads();
+    }
   }
 }
 template <int KP>
-__global__ void __launch_bounds__(kThreads) k_to_colmajor(int n, int s, const double* __restrict__ src, double* __restrict__ dst) {
-  using T = TransposeTile<KP>;
-  __shared__ T t;
-  for (int r0 = blockIdx.x * kTrRows; r0 < n; r0 += gridDim.x * kTrRows) {
-    const int rows = min(kTrRows, n - r0);
-    for (int q = threadIdx.x; q < rows * KP; q += kThreads) t.v[(q % KP) * T::LD + q / KP] = src[(size_t)r0 * KP + q];
-    __syncthreads();
-    for (int q = threadIdx.x; q < s * kTrRows; q += kThreads) {
-      const int j = q / kTrRows, r = q % kTrRows;
-      if (r < rows) dst[(size_t)j * n + r0 + r] = t.v[j * T::LD + r];
+__global__ void __launch_bounds__(kThreads)
+k_to_colmajor(int n, int s, const double* __restrict__ src, double* __restrict__ dst) {
+  if constexpr (KP < kTrMinKP) {
+    const size_t total = (size_t)n * s;
+    for (size_t q = blockIdx.x * (size_t)kThreads + threadIdx.x; q < total; q += (size_t)gridDim.x * kThreads) {
+      const size_t j = q / n, i = q % n;
+      dst[q] = src[i * KP + j];
     }
-    __syncthreads();
+  } else {
+    using T = TransposeTile<KP>;
+    __shared__ T t;
+    for (int r0 = blockIdx.x * kTrRows; r0 < n; r0 += gridDim.x * kTrRows) {
+      const int rows = min(kTrRows, n - r0);
+      for (int q = threadIdx.x; q < rows * KP; q += kThreads)
+        t.v[(q % KP) * T::LD + q / KP] = src[(size_t)r0 * KP + q];
+      __syncthreads();
+      for (int q = threadIdx.x; q < s * kTrRows; q += kThreads) {
+        const int j = q / kTrRows, r = q % kTrRows;
+        if (r < rows) dst[(size_t)j * n + r0 + r] = t.v[j * T::LD + r];
+      }
+      __syncthreads();
+    }
   }
 }
 
