@@ -673,10 +673,10 @@ void enqueue_product(mbpcg_ctx* h, const RowOps* ops, const double* X, double* Y
   } else if (h->prod64 == MBPCG_PRODUCT_CSR_TILED) {
     spmm_tiled(h->stream, dm.kp, dm.nb, dm.n, h->rp, h->av, h->plan, X, Y, h->part, dm.pstride, st,
                gram && !dm.mx_gram);
-    if (gram && dm.mx_gram) ops->gram_mx(h->stream, dm.nb_mx, dm.n, X, Y, nullptr, h->part, dm.pstride, st);
+    if (gram && dm.mx_gram) ops->gram_mx(h->stream, dm.nb_mx, dm.n, X, Y, nullptr, nullptr, h->part, dm.pstride, st);
   } else {
     ops->spmm(h->stream, dm.nb, dm.n, h->rp, h->ci, h->av, X, Y, h->part, dm.pstride, st, gram && !dm.mx_gram);
-    if (gram && dm.mx_gram) ops->gram_mx(h->stream, dm.nb_mx, dm.n, X, Y, nullptr, h->part, dm.pstride, st);
+    if (gram && dm.mx_gram) ops->gram_mx(h->stream, dm.nb_mx, dm.n, X, Y, nullptr, nullptr, h->part, dm.pstride, st);
   }
 }
 
@@ -706,7 +706,7 @@ void enqueue_mbpcg_setup(mbpcg_ctx* h) {
   enqueue_reduce(h, 3, nullptr);
   k_small_setup<<<1, 1, 0, h->stream>>>(h->st, h->red);
   ops->init(h->stream, dm.nb, n, h->s, h->U, h->Q, h->bs, h->X0, h->Xt, h->R, h->part, dm.pstride, h->st, !dm.mx);
-  if (dm.mx) ops->gram_mx(h->stream, dm.nb_mx, n, h->R, h->R, nullptr, h->part, dm.pstride, nullptr);
+  if (dm.mx) ops->gram_mx(h->stream, dm.nb_mx, n, h->R, h->R, nullptr, nullptr, h->part, dm.pstride, nullptr);
   enqueue_reduce(h, npack(kp), nullptr, dm.mx);
   launch_small_sigma(h->stream, kp, h->st, h->red, h->Sigma, h->SigmaInv);
   if (dm.mx_pw) ops->pw_mx(h->stream, dm.nb_mx, n, h->R, h->W, h->P, h->SigmaInv, nullptr, nullptr, 1);
@@ -740,9 +740,10 @@ void enqueue_mbpcg_body(mbpcg_ctx* h) {
   } else if (dm.mx) {
     ops->axpy_mx(h->stream, dm.nb_mx, n, h->P, h->Q, h->W, h->R, h->Xt, h->V, h->T, h->Xi, h->wdiag, h->part,
                  dm.pstride, h->st, h->rfree);
-    ops->gram_mx(h->stream, dm.nb_mx, n, h->V, h->V, nullptr, h->part, dm.pstride, h->st);
+    ops->gram_mx(h->stream, dm.nb_mx, n, h->V, h->V, nullptr, nullptr, h->part, dm.pstride, h->st);
     if (h->rfree && h->wdiag != nullptr)  // V^T D^2 V
-      ops->gram_mx(h->stream, dm.nb_mx, n, h->V, h->V, h->wdiag, h->part + npack(kp) + kp, dm.pstride, h->st);
+      ops->gram_mx(h->stream, dm.nb_mx, n, h->V, h->V, h->sqd, h->wdiag, h->part + npack(kp) + kp, dm.pstride,
+                   h->st);
   } else {
     ops->axpy(h->stream, dm.nb, n, h->P, h->Q, h->W, h->R, h->Xt, h->V, h->T, h->Xi, h->wdiag, h->part, dm.pstride,
               h->st, h->rfree);
@@ -772,8 +773,8 @@ void enqueue_mbpcg_exit(mbpcg_ctx* h) {
   const int kp = dm.kp, n = dm.n;
   if (h->rfree) ops->rsig(h->stream, dm.nb, n, h->V, h->W, h->Sigma, h->R, h->st);
   ops->ls_gram(h->stream, dm.nb, n, h->R, h->rhs, h->sqd, h->part, dm.pstride, !dm.mx);
-  if (dm.mx) {  // (D R)^T (D R) = R^T D^2 R; the other entries from their own partials
-    ops->gram_mx(h->stream, dm.nb_mx, n, h->R, h->R, h->wdiag, h->part, dm.pstride, nullptr);
+  if (dm.mx) {  // (D R)^T (D R); the other entries from their own partials
+    ops->gram_mx(h->stream, dm.nb_mx, n, h->R, h->R, h->sqd, h->wdiag, h->part, dm.pstride, nullptr);
     enqueue_reduce(h, npack(kp), nullptr, 1);
     enqueue_reduce(h, kp + 1, nullptr, 0, npack(kp));
   } else {

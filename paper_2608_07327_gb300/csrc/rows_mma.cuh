@@ -432,8 +432,9 @@ k_pw_mx(int n, const double* __restrict__ V, double* __restrict__ W, double* __r
 
 // ------------------------------------------------------------------------------------ Gram matrices
 
-// CTA partials of the upper triangle of X^T Y (Y = X when SYM), row i of X weighted by w_i when w is
-// given. A warp keeps its own column scales: the mma takes 16 view rows as its reduction index, so that a
+// CTA partials of the upper triangle of X^T Y (Y = X when SYM). WT: of X^T D^2 X,
+// with D in dw and as (D X)^T (D X) up to KP = 16, where that leaves one block to split (diffusion 77^3: 56 us
+// against 80 for (D^2 X)^T X), and D^2 in dw at KP = 32, where there are two anyway (FP64 products). A warp keeps its own column scales: the mma takes 16 view rows as its reduction index, so that a
 // lane holds the view columns g and g + 8 of 4 rows, as the left operand and as the right one alike. The
 // scales only grow; a tile that exceeds them (the first one, and then rarely: one bit of headroom) first
 // has the sums turned into FP64. KP = 32 is three problems of 16 columns (blockIdx.y: columns 0..15 with
@@ -441,9 +442,9 @@ k_pw_mx(int n, const double* __restrict__ V, double* __restrict__ W, double* __r
 constexpr int kMxDrainTiles = 8;    // 128 rows between two drains of the FP32 sums into int64
 constexpr int kMxFlushTiles = 16;   // 256 rows of 2^54 between two conversions of the int64 sums
 
-template <int KP, bool SYM>
+template <int KP, bool SYM, bool WT = false>
 __global__ void __launch_bounds__(kMxThreads, SYM && KP <= 16 ? 2 : 1)
-k_gram_mx(int n, const double* __restrict__ X, const double* __restrict__ Y, const double* __restrict__ w,
+k_gram_mx(int n, const double* __restrict__ X, const double* __restrict__ Y, const double* __restrict__ dw,
           double* __restrict__ part, int pstride, const SolveState* __restrict__ st) {
   constexpr int KV = 16, WARPS = kMxThreads / 32;
   if (st != nullptr && st->done) return;
@@ -518,10 +519,8 @@ k_gram_mx(int n, const double* __restrict__ X, const double* __restrict__ Y, con
         const size_t o = r * LD + g + 8 * c;
         const bool in = r < nv && (KP >= KV || o < nf);
         x[h][c] = in ? __ldg(X + o + xc) : 0.0;
-        if constexpr (!ONE) {
-          y[h][c] = in ? __ldg(Y + o + yc) : 0.0;
-          if (w != nullptr && in) x[h][c] *= __ldg(w + (o / KP));
-        }
+        if constexpr (!ONE) y[h][c] = in ? __ldg(Y + o + yc) : 0.0;
+        if constexpr (WT) x[h][c] *= in ? __ldg(dw + (o / KP)) : 0.0;
       }
     }
   };
