@@ -1544,15 +1544,13 @@ static int k_product_gram(int dense, int32_t n, const int32_t* rp, const int32_t
   const RowOps* ops = row_ops(dm.kp);
   cudaStream_t st = (cudaStream_t)stream;
   double* part = static_cast<double*>(scratch);
-  double* red = part + (size_t)dm.nbmax * dm.pstride;
   if (dense) {
     ops->dense(st, dm.nb_dense, n, A, P, AP, nullptr, nullptr);
     ops->gram(st, dm.nb, n, P, AP, part, dm.pstride, nullptr);
   } else {
     ops->spmm(st, dm.nb, n, rp, ci, av, P, AP, part, dm.pstride, nullptr, 1);
   }
-  launch_reduce(st, part, dm.nb, dm.pstride, red, npack(dm.kp), nullptr);
-  k_unpack_full<<<1, 256, 0, st>>>(red, dm.kp, s, G);
+  launch_reduce_gram(st, part, dm.nb, dm.pstride, s, G);
   CUDA_TRY(cudaGetLastError());
   return MBPCG_OK;
 }
@@ -1571,11 +1569,9 @@ int mbpcg_k_spmm_gram_f32(int32_t n, const int32_t* row_ptr, const int32_t* col_
   apply_mixed(dm);
   cudaStream_t st = (cudaStream_t)stream;
   double* part = static_cast<double*>(scratch);
-  double* red = part + (size_t)dm.nbmax * dm.pstride;
   row_ops_f(dm.kp)->spmm(st, dm.nb, n, row_ptr, col_idx, vals, P, AP, nullptr, 0, nullptr, 0, 8);
   row_ops_f(dm.kp)->gram(st, dm.nb, n, P, AP, part, dm.pstride, nullptr);
-  launch_reduce(st, part, dm.nb, dm.pstride, red, npack(dm.kp), nullptr);
-  k_unpack_full<<<1, 256, 0, st>>>(red, dm.kp, s, G);
+  launch_reduce_gram(st, part, dm.nb, dm.pstride, s, G);
   CUDA_TRY(cudaGetLastError());
   return MBPCG_OK;
 }
@@ -1746,14 +1742,6 @@ void product_gram_shape(int n, int s, int* kp, int* nb, int* pstride) {
 }
 
 int set_last_error(int code, const char* msg) { return set_err(code, "%s", msg); }
-
-// G (s x s column-major, ld s) = the full symmetric matrix of a packed upper triangle.
-__global__ void k_unpack_full(const double* __restrict__ packed, int kp, int s, double* __restrict__ G) {
-  for (int q = threadIdx.x; q < s * s; q += blockDim.x) {
-    const int l = q % s, m = q / s;
-    G[q] = (l <= m) ? packed[pidx(l, m)] : packed[pidx(m, l)];
-  }
-}
 
 // Z = upper Cholesky factor of G (s x s, ld s); *status = 0 or 6 (breakdown).
 __global__ void k_chol_only(const double* __restrict__ G, int s, double* __restrict__ Z, int* __restrict__ status) {

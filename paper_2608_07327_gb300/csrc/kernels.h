@@ -293,7 +293,7 @@ void product_gram_shape(int n, int s, int* kp, int* nb, int* pstride);
 int set_last_error(int code, const char* msg);
 
 // kernel-level helpers for the component entry points (api.cu)
-__global__ void k_unpack_full(const double* packed, int kp, int s, double* G);
+void launch_reduce_gram(cudaStream_t st, const double* part, int nparts, int pstride, int s, double* G);
 __global__ void k_chol_only(const double* G, int s, double* Z, int* status);
 
 }  // namespace mbpcg

@@ -120,11 +120,9 @@ extern "C" int mbpcg_k_spmm_gram_noalloc(int32_t n, const int32_t* row_ptr, cons
   if (rc != MBPCG_OK) return rc;
   // Every partial slot the reduction reads (nb of them) is fully written by this call's product
   // kernel first, so nothing in the array has to start at zero.
-  double* red = scratch + (size_t)kMaxCtas * kSlot;
   cudaStream_t st = (cudaStream_t)stream;
   mbpcg::row_ops(kp)->spmm(st, nb, n, row_ptr, col_idx, vals, P, AP, scratch, kSlot, nullptr, 1);
-  mbpcg::launch_reduce(st, scratch, nb, kSlot, red, mbpcg::npack(kp), nullptr);
-  mbpcg::k_unpack_full<<<1, 256, 0, st>>>(red, kp, s, G);
+  mbpcg::launch_reduce_gram(st, scratch, nb, kSlot, s, G);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess)
     return mbpcg::set_last_error(MBPCG_ERR_CUDA, cudaGetErrorString(e));

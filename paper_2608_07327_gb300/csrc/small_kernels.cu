@@ -5,15 +5,15 @@
 
 namespace mbpcg {
 
-// One CTA of kReduceThreads per entry: thread t sums the partials p = t, t + kReduceThreads, ...,
-// each warp combines its lanes by a butterfly, and thread 0 adds the warp sums in warp order
-// (a fixed order: the same bits on every run).
-__global__ void __launch_bounds__(kReduceThreads)
-k_reduce(const double* __restrict__ part, int nparts, int pstride, double* __restrict__ out, int nent,
-         const SolveState* __restrict__ st) {
+namespace {
+
+// Entry e of the sums over nparts partials, by one CTA of kReduceThreads: thread t sums the partials p = t,
+// t + kReduceThreads, ..., each warp combines its lanes by a butterfly, and thread 0 adds the warp sums in warp
+// order (a fixed order: the same bits on every run). True in thread 0, with the sum; nowhere when st is done.
+__device__ __forceinline__ bool reduce_entry(const double* __restrict__ part, int nparts, int pstride, int e,
+                                             const SolveState* __restrict__ st, double& sum) {
   __shared__ double ws[kReduceThreads / 32];
-  const int e = blockIdx.x, tid = threadIdx.x;
-  if (e >= nent) return;
+  const int tid = threadIdx.x;
   // batches of kB partials per thread, all loads of a batch in flight together; the first batch
   // is loaded with the solve state (a skipped launch discards it), so the two L2 round trips
   // overlap. The adds keep the partials' order.
@@ -27,7 +27,7 @@ k_reduce(const double* __restrict__ part, int nparts, int pstride, double* __res
     }
   };
   load(tid);
-  if (st != nullptr && st->done) return;
+  if (st != nullptr && st->done) return false;
   double a = 0.0;
   for (int p0 = tid; p0 < nparts; p0 += kB * kReduceThreads) {
     if (p0 != tid) load(p0);
@@ -38,16 +38,41 @@ k_reduce(const double* __restrict__ part, int nparts, int pstride, double* __res
   for (int off = 16; off; off >>= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
   if ((tid & 31) == 0) ws[tid >> 5] = a;
   __syncthreads();
-  if (tid == 0) {
-    double t = ws[0];
-    for (int w = 1; w < kReduceThreads / 32; ++w) t += ws[w];
-    out[e] = t;
-  }
+  if (tid != 0) return false;
+  sum = ws[0];
+  for (int w = 1; w < kReduceThreads / 32; ++w) sum += ws[w];
+  return true;
+}
+
+}  // namespace
+
+__global__ void __launch_bounds__(kReduceThreads)
+k_reduce(const double* __restrict__ part, int nparts, int pstride, double* __restrict__ out, int nent,
+         const SolveState* __restrict__ st) {
+  const int e = blockIdx.x;
+  if (e >= nent) return;
+  double v;
+  if (reduce_entry(part, nparts, pstride, e, st, v)) out[e] = v;
 }
 
 void launch_reduce(cudaStream_t s, const double* part, int nparts, int pstride, double* out, int nent,
                    const SolveState* st) {
   k_reduce<<<nent, kReduceThreads, 0, s>>>(part, nparts, pstride, out, nent, st);
+}
+
+// The Gram of a component product: the sums of the packed upper triangle, both triangles of the leading s x s
+// block of it into G (column-major). A launch less than sums and then matrix (Poisson 120^2, s = 4: 14.4 -> 11 to 12
+// us for product and Gram).
+__global__ void __launch_bounds__(kReduceThreads)
+k_reduce_gram(const double* __restrict__ part, int nparts, int pstride, int s, double* __restrict__ G) {
+  int l, m;
+  punpack(blockIdx.x, l, m);  // (the packed index goes by columns: those below npack(s) are l <= m < s)
+  double v;
+  if (reduce_entry(part, nparts, pstride, blockIdx.x, nullptr, v)) G[l + m * s] = G[m + l * s] = v;
+}
+
+void launch_reduce_gram(cudaStream_t st, const double* part, int nparts, int pstride, int s, double* G) {
+  k_reduce_gram<<<npack(s), kReduceThreads, 0, st>>>(part, nparts, pstride, s, G);
 }
 
 __global__ void k_params(SolveState* st, double tol_rel, int maxit, int no_test, int restart, int s, int stag) {
