@@ -681,12 +681,13 @@ cudaLaunchConfig_t lc_config(int kp, int n, int zcap, cudaStream_t s, cudaLaunch
 
 }  // namespace
 
-// The line: FP64 FMAs of one iteration (the 16 SMs do about 47 thousand a microsecond, 8 to 14 us besides),
-// where both sides measured alike. us per iteration, launches against this kernel:
-//   Poisson, s = 1: n = 256 23.9 / 5.9, 16384 26.7 / 10.2; s = 2: 4096 26.3 / 8.9, 16384 30.3 / 19.2;
-//   s = 4: 256 31.8 / 8.5, 4096 31.8 / 15.5, 6400 33.1 / 21.2, 10000 (1.28 M) 34.5 / 28.9, 12100 (1.55 M) 34.8 / 33.4;
-//   s = 8: 256 32.8 / 13.8, 2025 (0.91 M) 33.8 / 24.8, 4096 (1.83 M) 33.7 / 38.6;
-//   27-point, s = 4: n = 1728 38.6 / 13.9, 5832 (1.21 M) 39.1 / 29.6; s = 8: 1728 (1.04 M) 37.5 / 28.7.
+// The line: FP64 FMAs of one iteration (the 16 SMs do about 47 thousand a microsecond, 6 to 14 us besides),
+// below which no size measured was slower. us per iteration, launches of the row kernels / this kernel:
+//   Poisson, s = 1: n = 256 23.9 / 5.9, 16384 26.7 / 10.2, 32761 27.1 / 16.1, 44100 30.4 / 21.3;
+//   s = 2: 4096 26.3 / 8.9, 16384 30.3 / 19.2, 25600 30.9 / 29.7; s = 4: 256 31.8 / 8.5, 4096 29.2 / 15.6,
+//   8100 29.8 / 24.7, 10000 (1.28 M) 34.1 / 29.0; s = 8: 256 32.8 / 13.8, 2025 (0.91 M) 34.1 / 25.1, 3025
+//   (1.35 M) 33.7 / 32.1, 4096 (1.83 M) 33.7 / 38.6; 27-point, s = 4: n = 1728 38.6 / 13.9, 5832 (1.21 M) 36.9 /
+//   29.6; s = 8: 1728 (1.04 M) 37.9 / 28.7, 2197 (1.33 M) 37.7 / 34.7.
 // From KP = 16 the k x k steps are larger than one warp's work (clusters of their own, small_warp.cu).
 bool loop_cluster_fits(int kp, int n, long long nnz) {
   if (kp > 8) return false;

@@ -907,21 +907,23 @@ __global__ void k_gen_u(int n, int s, unsigned long long seed, double* __restric
   }
 }
 
-// Column-major n x s (leading dimension n) <-> row-major n x KP with zero padding. From KP = 8 by tiles of
-// kTrRows rows turned in shared memory so that both sides move whole 128-byte lines: 27-point 96^3, KP = 16,
-// s = 16: 152 -> 37 us. Below, a thread per value: its strided side still fills 32-byte sectors together with
-// its neighbours' (diffusion 128^3 out of KP = 4, 2, 1: 23, 13, 9 us against 39, 33, 28 by tiles).
+// Column-major n x s (leading dimension n) <-> row-major n x KP with zero padding. TILED: tiles of kTrRows rows
+// turned in shared memory, so that both sides move whole 128-byte lines (27-point 96^3, KP = 16, s = 16: 152 ->
+// 37 us). Otherwise a thread per value, whose strided side fills 32-byte sectors together with its neighbours':
+// below KP = 8 (diffusion 128^3 out of KP = 4, 2, 1: 23, 13, 9 us against 39, 33, 28 by tiles) and for small
+// blocks, where tiles are too few (us by tiles / by values, out of the block: n KP = 2^17: 3.7 / 2.5; 2^17.8:
+// 2.4 / 2.9; 2^18: 3.0 / 2.9; 2^19: 2.7 / 4.3; 2^20: 4.2 / 6.6).
 constexpr int kTrRows = 64;
-constexpr int kTrMinKP = 8;
+inline bool tr_tiled(int kp, int n) { return kp >= 8 && (long long)n * kp >= 1 << 18; }
 template <int KP>
 struct TransposeTile {
   static constexpr int LD = kTrRows + 1;
   double v[KP * LD];  // v[j * LD + r]
 };
-template <int KP>
+template <int KP, bool TILED>
 __global__ void __launch_bounds__(kThreads)
 k_from_colmajor(int n, int s, const double* __restrict__ src, double* __restrict__ dst) {
-  if constexpr (KP < kTrMinKP) {
+  if constexpr (!TILED) {
     const size_t total = (size_t)n * KP;
     for (size_t q = blockIdx.x * (size_t)kThreads + threadIdx.x; q < total; q += (size_t)gridDim.x * kThreads) {
       const int j = (int)(q % KP);
@@ -943,10 +945,10 @@ k_from_colmajor(int n, int s, const double* __restrict__ src, double* __restrict
     }
   }
 }
-template <int KP>
+template <int KP, bool TILED>
 __global__ void __launch_bounds__(kThreads)
 k_to_colmajor(int n, int s, const double* __restrict__ src, double* __restrict__ dst) {
-  if constexpr (KP < kTrMinKP) {
+  if constexpr (!TILED) {
     const size_t total = (size_t)n * s;
     for (size_t q = blockIdx.x * (size_t)kThreads + threadIdx.x; q < total; q += (size_t)gridDim.x * kThreads) {
       const size_t j = q / n, i = q % n;
