@@ -156,6 +156,16 @@ inline int dense_rows(int n, int nb) {
   return ((rows + passes - 1) / passes + 3) / 4;
 }
 
+// 8-byte asynchronous copy of one thread (cp.async), for data that no bulk copy can take.
+__device__ __forceinline__ void cp_async_8(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
+}
+
+// One of the arrivals that `bar` counts, made when the copies this thread has issued by cp_async_8 are done.
+__device__ __forceinline__ void cp_async_mbar_arrive(uint64_t* bar) {
+  asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_addr(bar)) : "memory");
+}
+
 constexpr int kDenseThreads = kThreads + 32;  // 8 warps multiply, the last one issues the copies
 
 template <int KP, int TR>

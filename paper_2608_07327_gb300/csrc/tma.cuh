@@ -62,16 +62,6 @@ __device__ __forceinline__ void tma_load_1d(void* dst, const void* src, uint32_t
       : "memory");
 }
 
-// 8-byte asynchronous copy of one thread (cp.async), for data that no bulk copy can take.
-__device__ __forceinline__ void cp_async_8(void* dst, const void* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
-}
-
-// One of the arrivals that `bar` counts, made when the copies this thread has issued by cp_async_8 are done.
-__device__ __forceinline__ void cp_async_mbar_arrive(uint64_t* bar) {
-  asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_addr(bar)) : "memory");
-}
-
 // L2 policy for data read once per pass and too large for L2: its lines are the first to go, so
 // they do not push out data that is reused (createpolicy, sm_80+).
 __device__ __forceinline__ uint64_t l2_policy_evict_first() {
