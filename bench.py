@@ -219,22 +219,32 @@ def read_ceiling_gbs(stream, flush):
     return 4 * (1 << 28) / (statistics.median(ts) * 1e-3) / 1e9
 
 
-BODY_UNROLL = 4  # loop iterations per pass of the library's graph loop (the passes end on whole bodies)
+BODY_UNROLL = 8  # loop iterations per pass of the library's graph loop (the passes end on whole bodies)
+CLUSTER_ITERS = 64  # iterations per launch of the one-cluster loop of small CSR systems
 
 
-def launches_per_solve(info, dense, algo_cg, tc=False, mixed=False, cg_fused=False):
+def launches_per_solve(info, dense, algo_cg, tc=False, mixed=False, cg_fused=False, n=0, nnz=0, s=0):
     """Kernels of ours launched by one solve call (the counter of the graph the library builds). The
     tensor-core dense product is four kernels (column exponents, digits of P, MMAs, split sum); the
-    mixed-precision loop runs its Gram as a kernel of its own; dense CG runs one kernel per
-    iteration. The graph loop runs whole passes of BODY_UNROLL iterations, so up to BODY_UNROLL - 1
-    bodies after the stop launch and return at once: counted here as launched (an upper bound)."""
+    mixed-precision loop runs its Gram as a kernel of its own; dense CG runs one kernel per iteration, CSR CG
+    three. FP64 CSR systems run their loop in one cluster when they are small, and two or three Grams as kernels
+    of their own when they are large (n, nnz, s given). The graph loop runs whole passes of BODY_UNROLL iterations,
+    so up to BODY_UNROLL - 1 bodies after the stop launch and return at once: counted here as launched (an upper
+    bound)."""
     inner = info["restarts"] + 1
+    kp = 1 << max(s - 1, 0).bit_length()
+    setup, exit_, body = 8, 7, (8 if (dense or mixed) else 7)
     if algo_cg:
-        setup, exit_, body = 3, 5, (1 if cg_fused else 5)
-    else:
-        setup, exit_, body = 8, 7, (8 if (dense or mixed) else 7)
-        if tc:
-            setup, body = setup + 3, body + 3
+        setup, exit_, body = 3, 5, (1 if cg_fused else 3)
+    elif tc:
+        setup, body = setup + 3, body + 3
+    elif n and not (dense or mixed):
+        rows = -(-n // 16)  # of one of the 16 CTAs; half of its matrix entries have to fit beside the blocks
+        if (kp <= 8 and nnz * kp + n * kp * (2 * (kp // 2 + 1) + 5 * kp + 1) <= 1400000
+                and 48 * rows * kp + 4 * rows + 12 * nnz // 32 <= 200000):
+            return inner * (1 + setup + exit_ + 1) + info["iterations"] // CLUSTER_ITERS + 1
+        if kp >= 4 and n * kp >= 1 << 17:
+            setup, exit_, body = setup + 1, exit_ + 2, body + 1 + (kp >= 16 and n * kp >= 1 << 19)
     bodies = info["iterations"] + (BODY_UNROLL - 1) * inner
     return inner * (1 + setup + exit_) + body * bodies + (0 if algo_cg else 1)
 
@@ -674,7 +684,8 @@ def run_ours(args, world, rank, local):
             "roofline": roofline,
             "e2e": {"value": round(e2e_ms, 4), "unit": UNIT, "h2d_bytes_per_step": 8 * n + 8 * n * s,
                     "d2h_bytes_per_step": 8 * n + 200 * (info["restarts"] + 1)},
-            "gpu_launches": sum(launches_per_solve(i, dense, False, prec == mb.MBPCG_FP64_TC, mixed) for i in infos),
+            "gpu_launches": sum(launches_per_solve(i, dense, False, prec == mb.MBPCG_FP64_TC, mixed, n=n,
+                                                       nnz=0 if dense else A.nnz, s=s) for i in infos),
             "gpu_launches_cg": sum(launches_per_solve(i, dense, True, cg_fused=dense and n % 2 == 0 and n <= 16384)
                                    for i in cg_infos),
             "clocks": clk.summary(),
@@ -902,7 +913,8 @@ def run_serving(args, world, rank):
                "identical_results": bool(all(np.array_equal(a["x"], b["x"]) for a, b in zip(q_res, res[:m])))}
     statuses = [r["status"] for r in res]
     relres = max(r["info"]["relres_true"] for r in res)
-    launches = sum(launches_per_solve(r["info"], False, False) for r in res)
+    launches = sum(launches_per_solve(r["info"], False, False, n=q["n"], nnz=cache.get(q["kind"], q["m"]).nnz, s=q["s"])
+                   for q, r in zip(reqs, res))
     h2d = float(np.mean([cache.get(q["kind"], q["m"]).nnz * 12 + (q["n"] + 1) * 4 + q["n"] * 8 for q in reqs]))
     line = {
         "metric": "serving p99 latency (submit to result), continuous batching", "value": round(p99, 3),
@@ -977,7 +989,8 @@ def run_batch(args, world, rank):
     ms_batch, ms_solo = max_over_ranks([float(np.median(times["batch"])), float(np.median(times["solo"]))], world, dev)
     same = all(np.array_equal(a[0], b[0]) and a[1]["iterations"] == b[1]["iterations"] for a, b in zip(ref, got))
     iters = sum(info["iterations"] for _, info in got)
-    launches = sum(launches_per_solve(info, False, False) for _, info in got)
+    launches = sum(launches_per_solve(info, False, False, n=r["n"], nnz=cache.get(r["kind"], r["m"]).nnz, s=r["s"])
+                   for r, (_, info) in zip(reqs, got))
     h2d = sum(r["n"] * 8 for r in reqs)
     batch.close()
     for sv in solvers:
