@@ -227,7 +227,7 @@ def launches_per_solve(info, dense, algo_cg, tc=False, mixed=False, cg_fused=Fal
     """Kernels of ours launched by one solve call (the counter of the graph the library builds). The
     tensor-core dense product is four kernels (column exponents, digits of P, MMAs, split sum); the
     mixed-precision loop runs its Gram as a kernel of its own; dense CG runs one kernel per iteration, CSR CG
-    three. FP64 CSR systems run their loop in one cluster when they are small, and two or three Grams as kernels
+    three or four. FP64 CSR systems run their loop in one cluster when they are small, and two or three Grams as kernels
     of their own when they are large (n, nnz, s given). The graph loop runs whole passes of BODY_UNROLL iterations,
     so up to BODY_UNROLL - 1 bodies after the stop launch and return at once: counted here as launched (an upper
     bound)."""
@@ -235,7 +235,7 @@ def launches_per_solve(info, dense, algo_cg, tc=False, mixed=False, cg_fused=Fal
     kp = 1 << max(s - 1, 0).bit_length()
     setup, exit_, body = 8, 7, (8 if (dense or mixed) else 7)
     if algo_cg:
-        setup, exit_, body = 3, 5, (1 if cg_fused else 3)
+        setup, exit_, body = 3, 5, (1 if cg_fused else 4)
     elif tc:
         setup, body = setup + 3, body + 3
     elif n and not (dense or mixed):

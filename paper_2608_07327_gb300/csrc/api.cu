@@ -844,6 +844,12 @@ void enqueue_cg_setup(mbpcg_ctx* h) {
   k_small_cg_setup<<<1, 1, 0, h->stream>>>(h->st, h->red);
 }
 
+// The three sums of CSR CG in its product, but for long rows of a large system, whose entries live on L1: there the
+// product alone keeps more of them (us, sums apart / in the product): 27-point 40^3 14.6 / 12.8, 48^3 17.5 / 15.8,
+// 56^3 23.1 / 25.5, 72^3 49 / 55, 96^3 102 / 121; 7-point 60^3 12.9 / 12.4, 128^3 65 / 61 (with scaling 70 / 62);
+// apart costs a launch besides.
+bool cg_sums_in_product(const Dims& dm) { return dm.nnz <= 16LL * dm.n || dm.n <= 1 << 17; }
+
 void enqueue_cg_body(mbpcg_ctx* h) {
   const Dims& dm = h->dm;
   if (dm.cg_fused) {
@@ -853,7 +859,7 @@ void enqueue_cg_body(mbpcg_ctx* h) {
     return;
   }
   const RowOps* ops = row_ops(1);  // w = A u, u = r, and the sums
-  if (!dm.dense && h->prod64 == MBPCG_PRODUCT_CSR_GATHER) {
+  if (!dm.dense && h->prod64 == MBPCG_PRODUCT_CSR_GATHER && cg_sums_in_product(dm)) {
     ops->spmm_dots(h->stream, dm.nb, dm.n, h->rp, h->ci, h->av, h->r, h->w, h->wdiag, h->part, dm.pstride, h->st);
   } else {
     enqueue_product(h, ops, h->r, h->w, 0, h->st);

@@ -97,26 +97,30 @@ k_spmm_dots(int n, const int* __restrict__ rp, const int* __restrict__ ci, const
             const double* __restrict__ r, double* __restrict__ w, const double* __restrict__ wdiag,
             double* __restrict__ part, int pstride, const SolveState* __restrict__ st) {
   if (st->done) return;
-  __shared__ double red[3 * kThreads];
+  // one sum at a time in 2 KB, and r_i and D^2 read after the row: entries of long rows live on L1, which shared
+  // memory takes away, and on registers (27-point 96^3: 172 us with 6 KB and r_i held, 121 so)
+  __shared__ double red[kThreads];
   int r0, r1;
   row_range(n, r0, r1);
   double g = 0.0, dl = 0.0, nu = 0.0;
   for (int i = r0 + threadIdx.x; i < r1; i += kThreads) {
     double acc = 0.0;
-    const double ri = __ldg(r + i), wd = wdiag != nullptr ? __ldg(wdiag + i) : 1.0;
     const int pe = __ldg(rp + i + 1);
 #pragma unroll 4
     for (int p = __ldg(rp + i); p < pe; ++p) acc = fma(__ldg(av + p), __ldg(r + __ldg(ci + p)), acc);
     w[i] = acc;
+    const double ri = __ldg(r + i), wd = wdiag != nullptr ? __ldg(wdiag + i) : 1.0;
     g = fma(ri, ri, g);
     dl = fma(acc, ri, dl);
     nu = (wdiag != nullptr) ? fma(ri * wd, ri, nu) : fma(ri, ri, nu);
   }
-  red[threadIdx.x * 3] = g;
-  red[threadIdx.x * 3 + 1] = dl;
-  red[threadIdx.x * 3 + 2] = nu;
-  cta_tree_sum(red, kThreads, 3);
-  if (threadIdx.x < 3) part[(size_t)blockIdx.x * pstride + threadIdx.x] = red[threadIdx.x];
+  const double v[3] = {g, dl, nu};
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    red[threadIdx.x] = v[q];
+    cta_tree_sum(red, kThreads, 1);
+    if (threadIdx.x == 0) part[(size_t)blockIdx.x * pstride + q] = red[0];
+  }
 }
 
 // ------------------------------------------------------------------------------------------------
