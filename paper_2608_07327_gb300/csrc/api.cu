@@ -661,6 +661,11 @@ int finish_create(mbpcg_ctx* h) {
 
 // ------------------------------------------------------------------------------- graph building
 
+// Two columns, long rows, a large system: the Gram by tiles, with fewer registers asked of the rows that live on
+// L1 (27-point, KP = 2, us in registers / by tiles: 60^3 37 / 41, 72^3 77 / 81, 84^3 115 / 102, 96^3 168 / 153;
+// 7-point 128^3 76 / 88).
+bool spmm_by_tiles(const Dims& dm) { return dm.kp == 2 && dm.nnz > 16LL * dm.n && dm.n > 1 << 19; }
+
 void enqueue_product(mbpcg_ctx* h, const RowOps* ops, const double* X, double* Y, int gram, const SolveState* st) {
   const Dims& dm = h->dm;
   if (dm.dense && dm.tc) {
@@ -675,7 +680,8 @@ void enqueue_product(mbpcg_ctx* h, const RowOps* ops, const double* X, double* Y
                gram && !dm.mx_gram);
     if (gram && dm.mx_gram) ops->gram_mx(h->stream, dm.nb_mx, dm.n, X, Y, nullptr, nullptr, h->part, dm.pstride, st);
   } else {
-    ops->spmm(h->stream, dm.nb, dm.n, h->rp, h->ci, h->av, X, Y, h->part, dm.pstride, st, gram && !dm.mx_gram);
+    ops->spmm(h->stream, dm.nb, dm.n, h->rp, h->ci, h->av, X, Y, h->part, dm.pstride, st,
+              gram && !dm.mx_gram ? (spmm_by_tiles(dm) ? 2 : 1) : 0);
     if (gram && dm.mx_gram) ops->gram_mx(h->stream, dm.nb_mx, dm.n, X, Y, nullptr, nullptr, h->part, dm.pstride, st);
   }
 }

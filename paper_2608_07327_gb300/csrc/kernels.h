@@ -26,7 +26,7 @@ inline cudaError_t ensure_dynamic_smem(K* func, size_t bytes) {
 struct RowOps {
   int kp;
   void (*spmm)(cudaStream_t, int nb, int n, const int* rp, const int* ci, const double* av, const double* P,
-               double* Q, double* part, int pstride, const SolveState* st, int gram);
+               double* Q, double* part, int pstride, const SolveState* st, int gram);  // gram 2: by tiles (KP = 2)
   // one column: the CG's w = A r with the CTA partials of k_cg_dots
   void (*spmm_dots)(cudaStream_t, int nb, int n, const int* rp, const int* ci, const double* av, const double* r,
                     double* w, const double* wdiag, double* part, int pstride, const SolveState* st);

@@ -16,7 +16,7 @@ namespace mbpcg {
 // when GRAM, the CTA partials of the upper triangle of P^T Q (the Gram that defines Xi), so that
 // A P is never read back. Threads own CPT consecutive columns of a row; the row of P that a
 // nonzero selects is KP*8 contiguous bytes, read with 16-byte vector loads.
-template <int KP, bool GRAM>
+template <int KP, bool GRAM, bool TILES = false>
 __global__ void __launch_bounds__(kThreads)
 k_spmm(int n, const int* __restrict__ rp, const int* __restrict__ ci, const double* __restrict__ av,
        const double* __restrict__ P, double* __restrict__ Q, double* __restrict__ part, int pstride,
@@ -26,8 +26,9 @@ k_spmm(int n, const int* __restrict__ rp, const int* __restrict__ ci, const doub
   if (st != nullptr && st->done) return;
   // A thread that has whole rows (KP <= 4) sums the Gram's terms of its rows in registers: KP (KP + 1) / 2 FMAs
   // a row and no barrier (diffusion 128^3, KP = 4: 148 us with the Gram against 167 by tiles; 129 us of
-  // the FP64 pipe; KP = 2 89 -> 77, KP = 1 59 -> 50; Poisson 160^2, KP = 4 11.5 -> 9.0).
-  constexpr bool kRegs = C::TPR == 1;
+  // the FP64 pipe; KP = 2 89 -> 77, KP = 1 59 -> 50; Poisson 160^2, KP = 4 11.5 -> 9.0);
+  // TILES keeps the tiles where they are the faster ones (spmm_by_tiles).
+  constexpr bool kRegs = C::TPR == 1 && !TILES;
   __shared__ __align__(16) double Xs[GRAM && !kRegs ? C::ROWS * KP : 2];
   __shared__ __align__(16) double Ys[GRAM && !kRegs ? C::ROWS * KP : 2];
   __shared__ __align__(16) double red[GRAM ? (kRegs ? C::NPACK * kThreads : G::RED) : 2];

@@ -33,3 +33,23 @@ def test_cg_after_ten_iterations(orc, name, factory, precond):
     xo, io = orc.cg_cgear(A, b, precond=precond, tol=1e-14, maxit=10)
     assert info["iterations"] == io["iterations"] == 10 and np.array_equal(x, y)
     assert np.linalg.norm(x - xo) <= 1e-9 * np.linalg.norm(xo)
+
+
+def test_two_columns_with_long_rows(orc):
+    """The product's Gram by tiles (more than 2^19 rows of more than 16 entries, s = 2): the state after one
+    iteration. Sums of n <= 532,000 terms, off by n 2^-53 = 6e-11 at worst on either side: 1e-9."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2608_07327_gb300 as mb
+    A = wl.stencil27(81, 2)
+    assert A.n > 1 << 19 and A.nnz > 16 * A.n
+    b, U = wl.rhs(A.n, 0), wl.initial_block(A.n, 2, 1)
+    sv = mb.Solver(A, s=2)
+    try:
+        got, st = sv.run_iterations(b, U, 1)
+    finally:
+        sv.close()
+    ref, st_o = orc.mbpcg_state(A, b, U, 1)
+    assert st == st_o == 0
+    for key in ("X0", "Xt", "R", "W", "P", "Sigma"):
+        assert np.abs(got[key] - ref[key]).max() <= 1e-9 * np.abs(ref[key]).max(), key
