@@ -167,6 +167,9 @@ __device__ __forceinline__ bool lc_factor(LcShared<KP>& sm, int s) {
   for (int j = 0; j < KP; ++j)
     if (j < s) mb = max(mb, __double_as_longlong(sm.S[j * KP + j]));
   const long long thr = __double_as_longlong(64.0 * DBL_EPSILON * __longlong_as_double(mb));
+  // Every thread has read the diagonal before step 0 changes it (at KP = 8 by two warps): one threshold, so
+  // one decision, in all threads and all CTAs.
+  kk_sync<KP>();
   bool bad = false;
   if (kt < KP && kt >= s) sm.d[kt] = sm.inv[kt] = 1.0;
   double linv = 1.0;  // 1/d of row a
