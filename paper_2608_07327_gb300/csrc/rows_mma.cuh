@@ -37,7 +37,8 @@
 //
 // Widths. The row products see the block as rows of KV = max(KP, 8) columns and a Gram as rows of 16: for
 // a narrower block several rows make one, with the k x k matrix repeated on the diagonal (the diagonal
-// blocks of the Gram summed).
+// blocks of the Gram summed). Every row of the block keeps a scale of its own: neighbouring unknowns may be in
+// different units, and a row 10^6 below its neighbour would lose 20 bits to a common one.
 //
 // A group that holds an infinity or a NaN has E = 0x7FF, and what is formed from it is NaN. A group below
 // 2^-958 counts as zero (the solver squares norms: it can use nothing below 2^-511).
@@ -203,7 +204,7 @@ __device__ void mx_load_matrix(F src, MxMatrix<KP>& M) {
   }
 }
 
-// A warp's 16 view rows of a block: digits, and the scale exponents of this lane's two rows.
+// A warp's 16 view rows of a block: digits, and the scale exponents of the two rows whose columns this lane has.
 template <int KP>
 struct MxTile {
   using W = MxRows<KP>;
@@ -218,7 +219,9 @@ struct MxTile {
 #pragma unroll
       for (int c = 0; c < W::NB; ++c) m = max(m, max(mx_exponent(v[c][r].x), mx_exponent(v[c][r].y)));
       m = max(m, __shfl_xor_sync(kMxAll, m, 1));
-      e[r] = max(m, __shfl_xor_sync(kMxAll, m, 2));
+      // at KP = 4 lanes t = 0, 1 hold one row of the block and t = 2, 3 the next one, here and in the results
+      if constexpr (KP >= 8) m = max(m, __shfl_xor_sync(kMxAll, m, 2));
+      e[r] = m;
 #pragma unroll
       for (int c = 0; c < W::NB; ++c) {
         uint32_t d[kMxDigits];

@@ -1,0 +1,84 @@
+"""The row products of the tensor-core passes (csrc/rows_mma.cuh) keep the precision of FP64 rows: measured on the
+state itself, without the k x k steps that made its factors. After one iteration X~ = P T with P = W of the set-up,
+and W = R Sigma^-1 after the set-up; the small factor is fitted to all rows in extended precision, and what a
+row is off from the fitted product is the row product's own error."""
+import numpy as np
+import pytest
+
+import workloads as wl
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+LD = np.longdouble
+U53 = 2.0 ** -53
+
+
+@pytest.fixture(scope="module")
+def mb():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2608_07327_gb300 as mb
+    mb.lib()
+    return mb
+
+
+def product(X, M):
+    """X M in extended precision."""
+    return sum(X[:, l:l + 1].astype(LD) * M[l:l + 1].astype(LD) for l in range(X.shape[1]))
+
+
+def solve_ld(G, B):
+    """G^-1 B by Gaussian elimination in extended precision (G small, positive definite)."""
+    G, B = G.astype(LD).copy(), B.astype(LD).copy()
+    k = len(G)
+    for j in range(k):
+        for i in range(j + 1, k):
+            f = G[i, j] / G[j, j]
+            G[i, j:] -= f * G[j, j:]
+            B[i] -= f * B[j]
+    for j in range(k - 1, -1, -1):
+        B[j] = (B[j] - (G[j, j + 1:, None] * B[j + 1:]).sum(0)) / G[j, j]
+    return B
+
+
+def fit(X, Y):
+    """The M that minimises |X M - Y|, columns of X brought to like size first."""
+    c = np.sqrt((X.astype(LD) ** 2).sum(0))
+    Xs = X / c
+    return solve_ld(product(Xs.T, Xs), product(Xs.T, Y)) / c[:, None]
+
+
+def scaled_grid(m, c):
+    """D (I + 0.05 L) D with L the five-point Laplacian on m x m and D alternating 1 and c: two unknowns
+    per cell in different units."""
+    L = wl.poisson2d(m)
+    d = np.where(np.arange(L.n) % 2 == 0, 1.0, c)
+    rows = np.repeat(np.arange(L.n), np.diff(L.row_ptr))
+    val = 0.05 * L.val
+    val[rows == L.col_idx] += 1.0
+    return wl.CSR(L.n, L.row_ptr, L.col_idx, val * d[rows] * d[L.col_idx])
+
+
+def states(mb, A, b, U, s, precond, iters):
+    sv = mb.Solver(A, s=s, precond=precond)
+    try:
+        return [sv.run_iterations(b, U, m)[0] for m in iters]
+    finally:
+        sv.close()
+
+
+@pytest.mark.parametrize("s", [3, 4])
+def test_neighbouring_rows_of_different_size(mb, s):
+    """Each entry within s^2 2^-53 of its row's largest value times its column's: what s FMAs of FP64 may be off
+    (each by 2^-53 of a partial sum of at most s such terms)."""
+    A = scaled_grid(183, 1e6)
+    n = A.n
+    assert n * 4 >= 1 << 17
+    z, one = states(mb, A, wl.rhs(n, 0), wl.initial_block(n, s, 1), s, 0, (0, 1))
+    big = np.abs(z["P"]).max(1, keepdims=True)
+    assert big.max() > 1e4 * big.min()  # the rows do differ
+    P, X = z["P"] / big, one["Xt"] / big
+    T = fit(P, X)
+    err = np.abs(product(P, T) - X).max(0) / np.abs(T).max(0)
+    assert (err <= s * s * U53).all(), err
