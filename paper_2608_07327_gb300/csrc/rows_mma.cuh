@@ -27,13 +27,16 @@
 // integer (|X| <= 2^B: the group's largest value keeps all its bits, any other loses what lies below
 // 2^-(B+1) of the scale), and X in 7 base-256 digits: six of -128..127 (X plus 128 in every digit, minus
 // 128 digit by digit) and a leading one of at most 2^(B-48), all exact in FP16. Digit pairs (t, u) are kept
-// for t + u <= 6 (28 products); what is dropped is random and below 2^-56 of the two scales at B = 56.
+// for t + u <= 6 (28 products); what is dropped is random, about 2^-58 of the two scales for each root of
+// a term at B = 57. (At B = 56 it is four times, at B = 55 sixteen times that: V zeta^-1 at KP = 32 was off by
+// 8e-17 and 2.6e-16 of its norm, the FP64 pass by 5.2e-17 and B = 57 by 5.1e-17; at B = 57 no product of any
+// width was further off than the FP64 pass on the Poisson, diffusion and 27-point systems, in an emulation.)
 // (With one side's digits 0..255, two operations fewer per pair of digits, what is dropped has a mean
 // that is the same for every row of a column: a smooth error, which an elliptic operator magnifies. The
 // state after 8 iterations of the 27-point stencil was 100 times further off.)
-//   A level sum S_L = sum_{t+u=L} sum_l is exact in the FP32 accumulator: below (2 * 2^15 + 5 * 2^14) * 16 <
-// 2^22 in the row products at B = 56, and 7 * 2^14 * 32 < 2^22 at the B = 55 of KP = 32; below 7 * 2^14 * 128
-// rows < 2^24 in a Gram (B = 55) between two drains.
+//   A level sum S_L = sum_{t+u=L} sum_l is exact in the FP32 accumulator: within 2^18 * 16 = 2^22 (level 0) and
+// (2 * 2^16 + 5 * 2^14) * 16 < 2^22 over one mma step of a row product at B = 57 (KP = 32 takes the levels of its
+// two steps out one after the other); below 7 * 2^14 * 128 rows < 2^24 in a Gram (B = 55) between two drains.
 //
 // Widths. The row products see the block as rows of KV = max(KP, 8) columns and a Gram as rows of 16: for
 // a narrower block several rows make one, with the k x k matrix repeated on the diagonal (the diagonal
@@ -145,7 +148,7 @@ struct MxRows {
   static constexpr int REP = KV / KP;  // rows of the block in a view row
   static constexpr int NB = KV / 8;
   static constexpr int KS = KV < 16 ? 1 : KV / 16;  // mma steps over the reduction index
-  static constexpr int B = KP >= 32 ? 55 : 56;
+  static constexpr int B = 57;
 };
 
 // A k x k matrix ready for the row products: the digits of each column in the fragment order of the
@@ -158,24 +161,24 @@ struct MxMatrix {
 };
 
 // The accumulators of a row product start at 3 2^22, whose last bit is worth 1: their bits then count the
-// level sum, which stays below 2^22 (two mma steps of 2^21).
+// level sum, which stays within 2^22 over one mma step. Level 6 starts 128 higher, which rounds it to level 5.
 constexpr uint32_t kMxStart = 0x4B400000u;
 
-// Weighted sum of the 7 levels' accumulators as integers, in units of 2^54 of the digits' product
-// (level L weighs 2^(8 (12 - L))), with the start values' share kMxStartSum, modulo 2^64: the total is
-// below 16 * 2^112 2^-54 = 2^62.
+// Weighted sum of the 7 levels' accumulators as integers, in units of 2^56 of the digits' product
+// (level L weighs 2^(8 (12 - L))), with the start values' share kMxStartSum, modulo 2^64: a step's total is
+// below 16 * 2^114 2^-56 = 2^62, that of two steps below 2^63 (the largest X is 2^57 - 2^4).
 __device__ __forceinline__ unsigned long long mx_levels(const float (&d)[kMxDigits][4], int q) {
-  unsigned long long r = __float_as_uint(d[6][q]) >> 6;
-  asm("mad.wide.u32 %0, %1, 4, %0;" : "+l"(r) : "r"(__float_as_uint(d[5][q])));
-  asm("mad.wide.u32 %0, %1, 1024, %0;" : "+l"(r) : "r"(__float_as_uint(d[4][q])));
-  asm("mad.wide.u32 %0, %1, 262144, %0;" : "+l"(r) : "r"(__float_as_uint(d[3][q])));
-  asm("mad.wide.u32 %0, %1, 67108864, %0;" : "+l"(r) : "r"(__float_as_uint(d[2][q])));
-  r += ((unsigned long long)((__float_as_uint(d[1][q]) << 2) + (__float_as_uint(d[0][q]) << 10))) << 32;
+  unsigned long long r = __float_as_uint(d[6][q]) >> 8;
+  r += __float_as_uint(d[5][q]);
+  asm("mad.wide.u32 %0, %1, 256, %0;" : "+l"(r) : "r"(__float_as_uint(d[4][q])));
+  asm("mad.wide.u32 %0, %1, 65536, %0;" : "+l"(r) : "r"(__float_as_uint(d[3][q])));
+  asm("mad.wide.u32 %0, %1, 16777216, %0;" : "+l"(r) : "r"(__float_as_uint(d[2][q])));
+  r += ((unsigned long long)(__float_as_uint(d[1][q]) + (__float_as_uint(d[0][q]) << 8))) << 32;
   return r;
 }
 constexpr unsigned long long kMxStartSum =
-    (unsigned long long)(kMxStart >> 6) + (unsigned long long)kMxStart * (4ull + 1024ull + 262144ull + 67108864ull) +
-    ((unsigned long long)(uint32_t)((kMxStart << 2) + (kMxStart << 10)) << 32);
+    (unsigned long long)(kMxStart >> 8) + (unsigned long long)kMxStart * (1ull + 256ull + 65536ull + 16777216ull) +
+    ((unsigned long long)(uint32_t)(kMxStart + (kMxStart << 8)) << 32);
 
 // Fills M from src(l, j) (KP x KP; all threads; the caller synchronises before and after).
 template <int KP, typename F>
@@ -235,13 +238,14 @@ struct MxTile {
   // Columns 8 nb + 2 t, + 1 of the two rows times M: y[r].
   __device__ __forceinline__ void times(const MxMatrix<KP>& M, int nb, double2 (&y)[2]) const {
     const int lane = threadIdx.x & 31;
-    float d[kMxDigits][4];
+    unsigned long long sum[4] = {0ull, 0ull, 0ull, 0ull};
 #pragma unroll
-    for (int L = 0; L < kMxDigits; ++L)
+    for (int ks = 0; ks < W::KS; ++ks) {
+      float d[kMxDigits][4];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) d[L][q] = __uint_as_float(kMxStart);
+      for (int L = 0; L < kMxDigits; ++L)
 #pragma unroll
-    for (int ks = 0; ks < W::KS; ++ks)
+        for (int q = 0; q < 4; ++q) d[L][q] = __uint_as_float(kMxStart + (L == kMxDigits - 1 ? 128u : 0u));
 #pragma unroll
       for (int u = 0; u < kMxDigits; ++u) {
         const uint2 b = M.b[u][ks][nb][lane];
@@ -251,12 +255,15 @@ struct MxTile {
           else mx_mma8(d[t + u], a[t], b.x);
         }
       }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) sum[q] += mx_levels(d, q) - kMxStartSum;
+    }
     const int j = (8 * nb + 2 * (lane & 3)) % KP;
     double v[4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const int f = M.e[j + (q & 1)], er = e[q >> 1];
-      v[q] = mx_double((long long)(mx_levels(d, q) - kMxStartSum), er + f - 2044 - 2 * W::B + 54);
+      v[q] = mx_double((long long)sum[q], er + f - 2044 - 2 * W::B + 56);
       if (max(f, er) == 0x7FF) v[q] = mx_nan();
     }
     y[0] = make_double2(v[0], v[1]);

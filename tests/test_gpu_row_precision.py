@@ -46,7 +46,11 @@ def fit(X, Y):
     """The M that minimises |X M - Y|, columns of X brought to like size first."""
     c = np.sqrt((X.astype(LD) ** 2).sum(0))
     Xs = X / c
-    return solve_ld(product(Xs.T, Xs), product(Xs.T, Y)) / c[:, None]
+
+    def gram(Z):
+        return np.stack([(Xs[:, l:l + 1] * Z).sum(0) for l in range(X.shape[1])])
+
+    return solve_ld(gram(Xs), gram(Y.astype(LD))) / c[:, None]
 
 
 def scaled_grid(m, c):
@@ -82,3 +86,22 @@ def test_neighbouring_rows_of_different_size(mb, s):
     T = fit(P, X)
     err = np.abs(product(P, T) - X).max(0) / np.abs(T).max(0)
     assert (err <= s * s * U53).all(), err
+
+
+@pytest.mark.parametrize("name,factory,s,precond", [
+    ("stencil26_s8", lambda: wl.stencil27(26, 1), 8, 0),
+    ("diffusion26_s16_jacobi", lambda: wl.diffusion3d(26, 2), 16, 1),
+    ("poisson92_s23", lambda: wl.poisson2d(92), 23, 0),
+    ("stencil21_s32", lambda: wl.stencil27(21, 3), 32, 0),
+    ("diffusion21_s32_jacobi", lambda: wl.diffusion3d(21, 4), 32, 1),
+])
+def test_products_are_off_by_little_more_than_their_rounding(mb, name, factory, s, precond):
+    """Root mean square of the errors of W = R Sigma^-1 and X~ = P T against that of the values. Rounding the result
+    to FP64 gives 0.43 x 2^-53 and splitting into digits adds a tenth of that; the sums of an FP64 pass are off by
+    more the more columns they have. The bound is 2^-53."""
+    A = factory()
+    assert A.n * mb.mbpcg_k_padded_width(s) >= 1 << 17
+    z, one = states(mb, A, wl.rhs(A.n, 0), wl.initial_block(A.n, s, 1), s, precond, (0, 1))
+    for X, Y in ((z["R"], z["W"]), (z["W"], one["Xt"])):
+        E = product(X, fit(X, Y)) - Y
+        assert np.sqrt((E ** 2).sum() / (Y.astype(LD) ** 2).sum()) <= U53
