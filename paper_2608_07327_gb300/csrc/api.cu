@@ -668,6 +668,7 @@ bool spmm_by_tiles(const Dims& dm) { return dm.kp == 2 && dm.nnz > 16LL * dm.n &
 
 void enqueue_product(mbpcg_ctx* h, const RowOps* ops, const double* X, double* Y, int gram, const SolveState* st) {
   const Dims& dm = h->dm;
+  const double* bal = h->wdiag == nullptr ? h->diag : nullptr;  // balances the Gram's rows; a scaled A has ones there
   if (dm.dense && dm.tc) {
     // the loop's product reads P, whose column exponents the W/P update has already formed
     oz_product(h->stream, dm.n, dm.kp, dm.sms, h->oz_a, h->oz_ea, X, h->oz_p, h->oz_ep, h->oz_q, Y, &h->st->kerr, st,
@@ -678,11 +679,11 @@ void enqueue_product(mbpcg_ctx* h, const RowOps* ops, const double* X, double* Y
   } else if (h->prod64 == MBPCG_PRODUCT_CSR_TILED) {
     spmm_tiled(h->stream, dm.kp, dm.nb, dm.n, h->rp, h->av, h->plan, X, Y, h->part, dm.pstride, st,
                gram && !dm.mx_gram);
-    if (gram && dm.mx_gram) ops->gram_mx(h->stream, dm.nb_mx, dm.n, X, Y, nullptr, nullptr, h->part, dm.pstride, st);
+    if (gram && dm.mx_gram) ops->gram_mx(h->stream, dm.nb_mx, dm.n, X, Y, nullptr, bal, h->part, dm.pstride, st);
   } else {
     ops->spmm(h->stream, dm.nb, dm.n, h->rp, h->ci, h->av, X, Y, h->part, dm.pstride, st,
               gram && !dm.mx_gram ? (spmm_by_tiles(dm) ? 2 : 1) : 0);
-    if (gram && dm.mx_gram) ops->gram_mx(h->stream, dm.nb_mx, dm.n, X, Y, nullptr, nullptr, h->part, dm.pstride, st);
+    if (gram && dm.mx_gram) ops->gram_mx(h->stream, dm.nb_mx, dm.n, X, Y, nullptr, bal, h->part, dm.pstride, st);
   }
 }
 

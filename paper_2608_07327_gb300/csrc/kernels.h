@@ -60,7 +60,7 @@ struct RowOps {
   void (*pw_pre)(cudaStream_t, int n, const double* VZi, const double* PZt, double* W, double* P, const SolveState* st,
                  int* emax);
   // the row passes on the tensor cores (rows_mma.cuh; KP >= 4): the Gram X^T Y (Y = X: X^T D^2 X with
-  // D and D^2, or NULL), the block update without its Gram, the W/P update
+  // D and D^2, or NULL; otherwise d2 is the diagonal that balances the rows, or NULL), the block update without its Gram, the W/P update
   void (*gram_mx)(cudaStream_t, int nb, int n, const double* X, const double* Y, const double* d, const double* d2,
                   double* part, int pstride, const SolveState* st);
   void (*axpy_mx)(cudaStream_t, int nb, int n, const double* P, const double* Q, const double* W, double* R,

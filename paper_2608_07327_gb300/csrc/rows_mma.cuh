@@ -36,7 +36,7 @@
 // state after 8 iterations of the 27-point stencil was 100 times further off.)
 //   A level sum S_L = sum_{t+u=L} sum_l is exact in the FP32 accumulator: within 2^18 * 16 = 2^22 (level 0) and
 // (2 * 2^16 + 5 * 2^14) * 16 < 2^22 over one mma step of a row product at B = 57 (KP = 32 takes the levels of its
-// two steps out one after the other); below 7 * 2^14 * 128 rows < 2^24 in a Gram (B = 55) between two drains.
+// two steps out one after the other); below (2 * 2^15 + 5 * 2^14) * 112 rows < 2^24 in a Gram (B = 56) between two drains.
 //
 // Widths. The row products see the block as rows of KV = max(KP, 8) columns and a Gram as rows of 16: for
 // a narrower block several rows make one, with the k x k matrix repeated on the diagonal (the diagonal
@@ -44,7 +44,7 @@
 // different units, and a row 10^6 below its neighbour would lose 20 bits to a common one.
 //
 // A group that holds an infinity or a NaN has E = 0x7FF, and what is formed from it is NaN. A group below
-// 2^-958 counts as zero (the solver squares norms: it can use nothing below 2^-511).
+// 2^-831 counts as zero (the solver squares norms: it can use nothing below 2^-511).
 #pragma once
 #include <cuda_fp16.h>
 #include <stdint.h>
@@ -59,21 +59,23 @@ namespace mbpcg {
 constexpr int kMxMinKP = 4;  // narrower blocks have too few FP64 operations per byte
 constexpr int kMxDigits = 7;
 constexpr int kMxThreads = 256;  // threads per CTA
-constexpr int kMxGramBits = 55;  // B of the Grams
+constexpr int kMxGramBits = 56;  // B of the Grams
 constexpr unsigned kMxAll = 0xffffffffu;
+constexpr int kMxTiny = 192;    // a group with a scale exponent below this one counts as zero
+constexpr int kMxNaN = 0x4000;  // scale exponent of a column of a Gram that is not finite
 
 __device__ __forceinline__ int mx_exponent(double x) { return (__double2hiint(x) >> 20) & 0x7FF; }
 
-// X of x in a group of scale exponent E (>= its own), to nearest (halves away from zero).
+// X of 2^o x (0 <= o < 128) in a group of scale exponent E (>= its own), to nearest (halves away from zero).
 template <int B>
-__device__ __forceinline__ long long mx_int(double x, int E) {
+__device__ __forceinline__ long long mx_int(double x, int E, int o = 0) {
   const int h = __double2hiint(x), e = (h >> 20) & 0x7FF;
   // 53 bits moved up to B + 1 (one below the unit), then down to the group's scale;
-  // shr.u64 gives 0 from 64 on, which a zero or subnormal x (e = 0) reaches since E >= 64
+  // shr.u64 gives 0 from 64 on, which a zero or subnormal x (e = 0) reaches since E >= 192
   const unsigned long long m = (((unsigned long long)(unsigned)((h & 0xFFFFF) | 0x100000) << 32) |
                                 (unsigned)__double2loint(x)) << (B - 52);
   unsigned long long r;
-  asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(m), "r"((E < 64 ? 4096 : E) - e));
+  asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(m), "r"((E < kMxTiny ? 4096 : E) - e - o));
   r = (r + 1) >> 1;
   const long long s = h >> 31;
   return (long long)(r ^ (unsigned long long)s) - s;
@@ -447,10 +449,14 @@ k_pw_mx(int n, const double* __restrict__ V, double* __restrict__ W, double* __r
 // against 80 for (D^2 X)^T X), and D^2 in dw at KP = 32, where there are two anyway (FP64 products). A warp keeps its own column scales: the mma takes 16 view rows as its reduction index, so that a
 // lane holds the view columns g and g + 8 of 4 rows, as the left operand and as the right one alike. The
 // scales only grow; a tile that exceeds them (the first one, and then rarely: one bit of headroom) first
-// has the sums turned into FP64. KP = 32 is three problems of 16 columns (blockIdx.y: columns 0..15 with
+// has the sums turned into FP64. 56 bits of the scale: with 55 the Grams of unscaled diffusion
+// were off by up to 1.5 times what FP64 sums are, with 56 by less than those on every system (in an emulation).
+// X^T Y of two blocks is P^T (A P). Where the diagonal of A varies, P is small where A P is large, and a scale over
+// the rows would lose what their product does not: the rows are balanced by r = half the exponent of a_ii (dw,
+// or NULL; to that of a_00, at most 63), 2^r X against 2^-r Y. (Two unknowns per point in units 10^6 apart, 16
+// columns, emulated: off by 2e-12 of the largest entry without and 1e-16 with it, FP64 sums by 1e-15.) KP = 32 is three problems of 16 columns (blockIdx.y: columns 0..15 with
 // themselves, with 16..31, and 16..31 with themselves).
-constexpr int kMxDrainTiles = 8;    // 128 rows between two drains of the FP32 sums into int64
-constexpr int kMxFlushTiles = 16;   // 256 rows of 2^54 between two conversions of the int64 sums
+constexpr int kMxDrainTiles = 7;  // 112 rows between two drains of the FP32 sums into FP64
 
 template <int KP, bool SYM, bool WT = false>
 __global__ void __launch_bounds__(kMxThreads, SYM && KP <= 16 ? 2 : 1)
@@ -458,6 +464,7 @@ k_gram_mx(int n, const double* __restrict__ X, const double* __restrict__ Y, con
           double* __restrict__ part, int pstride, const SolveState* __restrict__ st) {
   constexpr int KV = 16, WARPS = kMxThreads / 32;
   if (st != nullptr && st->done) return;
+  constexpr bool BAL = !SYM && KP >= KV;  // (a view row is a row of the block)
   __shared__ double red[WARPS][KV * KV];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
   // KP = 32: rows are 32 wide, this problem's columns start at xc (X) and yc (Y)
@@ -467,8 +474,9 @@ k_gram_mx(int n, const double* __restrict__ X, const double* __restrict__ Y, con
   const size_t step = (size_t)gridDim.x * WARPS * 16;
 
   float acc[kMxDigits][2][4];
-  long long sum[2][4];
   double f[2][4];
+  int rs[BAL ? 4 : 1];  // r of the tile's rows
+  const int e0 = BAL && dw != nullptr ? mx_exponent(__ldg(dw)) : 0;
   int ex[2] = {0, 0}, ey[2] = {0, 0};  // scale exponents of view columns g, g + 8
   auto zero = [&]() {
 #pragma unroll
@@ -478,7 +486,8 @@ k_gram_mx(int n, const double* __restrict__ X, const double* __restrict__ Y, con
 #pragma unroll
         for (int q = 0; q < 4; ++q) acc[L][b][q] = 0.f;
   };
-  // the FP32 sums into the int64 ones (units of 2^56 of the digits' product: level 5; level 6 rounded)
+  // the FP32 sums into FP64, over an integer in units of 2^56 of the digits' product (level 5; level 6 rounded):
+  // below 112 * 2^112 2^-56 < 2^63
   auto drain = [&]() {
 #pragma unroll
     for (int b = 0; b < 2; ++b)
@@ -487,36 +496,24 @@ k_gram_mx(int n, const double* __restrict__ X, const double* __restrict__ Y, con
         int s[kMxDigits];
 #pragma unroll
         for (int L = 0; L < kMxDigits; ++L) s[L] = __float2int_rn(acc[L][b][q]);
-        sum[b][q] += ((long long)s[0] << 40) + ((long long)s[1] << 32) + ((long long)s[2] << 24) +
-                     ((long long)s[3] << 16) + ((long long)s[4] << 8) + s[5] + ((s[6] + 128) >> 8);
-      }
-    zero();
-  };
-  // the int64 sums into FP64
-  auto flush = [&]() {
-#pragma unroll
-    for (int b = 0; b < 2; ++b)
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
+        const long long sum = ((long long)s[0] << 40) + ((long long)s[1] << 32) + ((long long)s[2] << 24) +
+                              ((long long)s[3] << 16) + ((long long)s[4] << 8) + s[5] + ((s[6] + 128) >> 8);
         // entry (g + 8 (q / 2), 8 b + 2 t + q % 2)
         const int el = ex[q >> 1];
         const int ej = __shfl_sync(kMxAll, SYM && KP <= KV ? ex[b] : ey[b], (2 * t + (q & 1)) * 4);
         bool ok;
-        const int k = el + ej - 2044 - 2 * kMxGramBits + 56;
-        double v = ll_to_double_scaled_rn(sum[b][q], k, ok);
-        if (!ok) v = ldexp(ll_to_double_rn(sum[b][q]), k);
-        f[b][q] += max(el, ej) == 0x7FF ? mx_nan() : v;
-        sum[b][q] = 0;
+        const int k = el + ej - 2044 - 2 * kMxGramBits + 56 - (BAL ? 126 : 0);
+        double v = ll_to_double_scaled_rn(sum, k, ok);
+        if (!ok) v = ldexp(ll_to_double_rn(sum), k);
+        f[b][q] += max(el, ej) == kMxNaN ? mx_nan() : v;
       }
+    zero();
   };
   zero();
 #pragma unroll
   for (int b = 0; b < 2; ++b)
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      sum[b][q] = 0;
-      f[b][q] = 0.0;
-    }
+    for (int q = 0; q < 4; ++q) f[b][q] = 0.0;
   // x[h][c]: row 2 t + (h & 1) + 8 (h >> 1) of the tile, view column g + 8 c
   constexpr bool ONE = SYM && KP <= KV;  // both operands from one block
   double x[4][2], y[ONE ? 1 : 4][2];
@@ -524,6 +521,8 @@ k_gram_mx(int n, const double* __restrict__ X, const double* __restrict__ Y, con
 #pragma unroll
     for (int h = 0; h < 4; ++h) {
       const size_t r = base + 2 * t + (h & 1) + 8 * (h >> 1);
+      if constexpr (BAL)
+        rs[h] = dw != nullptr && r < nv ? max(-63, min(63, (mx_exponent(__ldg(dw + r)) - e0) >> 1)) : 0;
 #pragma unroll
       for (int c = 0; c < 2; ++c) {
         const size_t o = r * LD + g + 8 * c;
@@ -534,25 +533,42 @@ k_gram_mx(int n, const double* __restrict__ X, const double* __restrict__ Y, con
       }
     }
   };
-  auto grow = [&](const auto& v, int (&e)[2], int (&ne)[2]) {
+  // X takes part as 2^(63 + r) X and Y as 2^(63 - r) Y
+  auto off = [&](int h, int sign) { return BAL ? 63 + sign * rs[BAL ? h : 0] : 0; };
+  auto grow = [&](const auto& v, int sign, const int (&e)[2], int (&ne)[2]) {
     bool over = false;
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
-      int m = max(max(mx_exponent(v[0][c]), mx_exponent(v[1][c])), max(mx_exponent(v[2][c]), mx_exponent(v[3][c])));
+      int m = 0;
+#pragma unroll
+      for (int h = 0; h < 4; ++h) m = max(m, mx_exponent(v[h][c]) + off(h, sign));
       m = max(m, __shfl_xor_sync(kMxAll, m, 1));
       m = max(m, __shfl_xor_sync(kMxAll, m, 2));
-      ne[c] = m > e[c] ? (m == 0x7FF ? m : min(m + 1, 0x7FE)) : e[c];
+      ne[c] = m > e[c] ? m + 1 : e[c];
       over |= ne[c] != e[c];
     }
     return over;
   };
-  auto split = [&](const auto& v, const int (&e)[2], uint32_t (&a)[kMxDigits][4]) {
+  // the new scales; an infinity or a NaN, whose exponent is the largest, is looked for only here
+  auto adopt = [&](const auto& v, const int (&ne)[2], int (&e)[2]) {
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      int bad = e[c] == kMxNaN;
+#pragma unroll
+      for (int h = 0; h < 4; ++h) bad |= mx_exponent(v[h][c]) == 0x7FF;
+      bad |= __shfl_xor_sync(kMxAll, bad, 1);
+      bad |= __shfl_xor_sync(kMxAll, bad, 2);
+      e[c] = bad ? kMxNaN : ne[c];
+    }
+  };
+  auto split = [&](const auto& v, int sign, const int (&e)[2], uint32_t (&a)[kMxDigits][4]) {
 #pragma unroll
     for (int hh = 0; hh < 2; ++hh)
 #pragma unroll
       for (int c = 0; c < 2; ++c) {
         uint32_t d[kMxDigits];
-        mx_digits(mx_int<kMxGramBits>(v[2 * hh][c], e[c]), mx_int<kMxGramBits>(v[2 * hh + 1][c], e[c]), d);
+        mx_digits(mx_int<kMxGramBits>(v[2 * hh][c], e[c], off(2 * hh, sign)),
+                  mx_int<kMxGramBits>(v[2 * hh + 1][c], e[c], off(2 * hh + 1, sign)), d);
 #pragma unroll
         for (int q = 0; q < kMxDigits; ++q) a[q][2 * hh + c] = d[q];
       }
@@ -562,22 +578,17 @@ k_gram_mx(int n, const double* __restrict__ X, const double* __restrict__ Y, con
   if (base < nv) load(base);
   for (; base < nv; base += step) {
     int nx[2], ny[2];
-    bool over = grow(x, ex, nx);
-    if constexpr (!ONE) over |= grow(y, ey, ny);
+    bool over = grow(x, 1, ex, nx);
+    if constexpr (!ONE) over |= grow(y, -1, ey, ny);
     if (__any_sync(kMxAll, over)) {
       drain();
-      flush();
       tiles = 0;
-      ex[0] = nx[0];
-      ex[1] = nx[1];
-      if constexpr (!ONE) {
-        ey[0] = ny[0];
-        ey[1] = ny[1];
-      }
+      adopt(x, nx, ex);
+      if constexpr (!ONE) adopt(y, ny, ey);
     }
     uint32_t a[kMxDigits][4], b[ONE ? 1 : kMxDigits][4];
-    split(x, ex, a);
-    if constexpr (!ONE) split(y, ey, b);
+    split(x, 1, ex, a);
+    if constexpr (!ONE) split(y, -1, ey, b);
     if (base + step < nv) load(base + step);
 #pragma unroll
     for (int u = 0; u < kMxDigits; ++u) {
@@ -588,15 +599,12 @@ k_gram_mx(int n, const double* __restrict__ X, const double* __restrict__ Y, con
         mx_mma16(acc[q + u][1], a[q], bu[1], bu[3]);
       }
     }
-    ++tiles;
-    if (tiles % kMxDrainTiles == 0) drain();
-    if (tiles == kMxFlushTiles) {
-      flush();
+    if (++tiles == kMxDrainTiles) {
+      drain();
       tiles = 0;
     }
   }
   drain();
-  flush();
 #pragma unroll
   for (int b = 0; b < 2; ++b)
 #pragma unroll

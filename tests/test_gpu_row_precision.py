@@ -105,3 +105,32 @@ def test_products_are_off_by_little_more_than_their_rounding(mb, name, factory, 
     for X, Y in ((z["R"], z["W"]), (z["W"], one["Xt"])):
         E = product(X, fit(X, Y)) - Y
         assert np.sqrt((E ** 2).sum() / (Y.astype(LD) ** 2).sum()) <= U53
+
+
+@pytest.mark.parametrize("s", [16, 25, 32])
+def test_product_gram_of_rows_in_different_units(mb, s):
+    """P is small where A P is large: P^T (A P) = G has terms of one size in rows whose factors are 10^6 apart. T = Xi
+    Sigma, fitted from X~ = P T, against G^-1 Sigma in extended precision. A sum of FP64 terms by at most 30 rows in
+    turn is off by 30 x 2^-53, the k x k steps add at most 8 s x 2^-53, and G^-1 magnifies both by its condition."""
+    scipy_linalg = pytest.importorskip("scipy.sparse.linalg")
+    A = scaled_grid(183, 1e6)
+    S = A.to_scipy().tocsc()
+    n, d = A.n, np.sqrt(S.diagonal())
+    assert n * mb.mbpcg_k_padded_width(s) >= 1 << 19
+    rows = wl.initial_block(n, s + 1, 1) / (d / d.min())[:, None]
+    b = rows[:, s].copy()
+    U = np.asfortranarray(scipy_linalg.splu(S).solve(b[:, None] - rows[:, :s]))
+    z, one = states(mb, A, b, U, s, 0, (0, 1))
+    P = z["W"].astype(LD)
+    Q = np.zeros_like(P)
+    for i in range(int(np.diff(A.row_ptr).max())):  # A P in extended precision, entry i of every row
+        at = A.row_ptr[:-1] + i
+        ok = at < A.row_ptr[1:]
+        Q[ok] += A.val[at[ok], None].astype(LD) * P[A.col_idx[at[ok]]]
+    assert np.abs(Q).max(1).max() > 1e5 * np.abs(P).max()  # the factors do differ
+    G = np.stack([(P[:, l:l + 1] * Q).sum(0) for l in range(s)])
+    ref = solve_ld(G, z["Sigma"])
+    T = fit(z["W"], one["Xt"])
+    cond = np.linalg.cond(G.astype(np.float64))
+    assert cond < 4
+    assert np.abs(T - ref).max() <= (30 + 8 * s) * U53 * cond * np.abs(ref).max()
