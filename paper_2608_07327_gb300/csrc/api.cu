@@ -716,7 +716,7 @@ void enqueue_mbpcg_setup(mbpcg_ctx* h) {
   if (dm.mx) ops->gram_mx(h->stream, dm.nb_mx, n, h->R, h->R, nullptr, nullptr, h->part, dm.pstride, nullptr);
   enqueue_reduce(h, npack(kp), nullptr, dm.mx);
   launch_small_sigma(h->stream, kp, h->st, h->red, h->Sigma, h->SigmaInv);
-  if (dm.mx_pw) ops->pw_mx(h->stream, dm.nb_mx, n, h->R, h->W, h->P, h->SigmaInv, nullptr, nullptr, 1);
+  if (dm.mx_pw) ops->pw_mx(h->stream, dm.nb_mx, n, h->R, h->W, h->P, h->SigmaInv, h->Sigma, nullptr, 1);
   else ops->pw(h->stream, dm.nb, n, h->R, h->W, h->P, h->SigmaInv, nullptr, nullptr, 1, dm.tc ? h->oz_ep : nullptr);
 }
 
@@ -745,7 +745,7 @@ void enqueue_mbpcg_body(mbpcg_ctx* h) {
     rowprod_tc(h->stream, n, kp, jb, 3, h->st, 0, &h->st->kerr);
     ops->axpy_pre(h->stream, dm.nb, n, Y0, Y1, Y2, h->W, h->R, h->Xt, h->V, h->wdiag, h->part, dm.pstride, h->st);
   } else if (dm.mx) {
-    ops->axpy_mx(h->stream, dm.nb_mx, n, h->P, h->Q, h->W, h->R, h->Xt, h->V, h->T, h->Xi, h->wdiag, h->part,
+    ops->axpy_mx(h->stream, dm.nb_mx, n, h->P, h->Q, h->W, h->R, h->Xt, h->V, h->T, h->Xi, h->red, h->wdiag, h->part,
                  dm.pstride, h->st, h->rfree);
     ops->gram_mx(h->stream, dm.nb_mx, n, h->V, h->V, nullptr, nullptr, h->part, dm.pstride, h->st);
     if (h->rfree && h->wdiag != nullptr)  // V^T D^2 V

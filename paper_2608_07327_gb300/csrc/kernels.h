@@ -60,12 +60,13 @@ struct RowOps {
   void (*pw_pre)(cudaStream_t, int n, const double* VZi, const double* PZt, double* W, double* P, const SolveState* st,
                  int* emax);
   // the row passes on the tensor cores (rows_mma.cuh; KP >= 4): the Gram X^T Y (Y = X: X^T D^2 X with
-  // D and D^2, or NULL; otherwise d2 is the diagonal that balances the rows, or NULL), the block update without its Gram, the W/P update
+  // D and D^2, or NULL; otherwise d2 is the diagonal that balances the rows, or NULL), the block update without its Gram (G: P^T A P, packed),
+  // the W/P update (setp: Z is the Cholesky factor Sigma of V)
   void (*gram_mx)(cudaStream_t, int nb, int n, const double* X, const double* Y, const double* d, const double* d2,
                   double* part, int pstride, const SolveState* st);
   void (*axpy_mx)(cudaStream_t, int nb, int n, const double* P, const double* Q, const double* W, double* R,
-                  double* Xt, double* V, const double* T, const double* Xi, const double* wdiag, double* part,
-                  int pstride, const SolveState* st, int rfree);
+                  double* Xt, double* V, const double* T, const double* Xi, const double* G, const double* wdiag,
+                  double* part, int pstride, const SolveState* st, int rfree);
   void (*pw_mx)(cudaStream_t, int nb, int n, const double* V, double* W, double* P, const double* Zinv,
                 const double* Z, const SolveState* st, int setp);
 };

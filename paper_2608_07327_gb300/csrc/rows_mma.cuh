@@ -37,6 +37,14 @@
 //   A level sum S_L = sum_{t+u=L} sum_l is exact in the FP32 accumulator: within 2^18 * 16 = 2^22 (level 0) and
 // (2 * 2^16 + 5 * 2^14) * 16 < 2^22 over one mma step of a row product at B = 57 (KP = 32 takes the levels of its
 // two steps out one after the other); below (2 * 2^15 + 5 * 2^14) * 112 rows < 2^24 in a Gram (B = 56) between two drains.
+//   A row product is off by 2^-58 or so of max_l |x_il| max_l |m_lj|, an FP64 sum by 2^-53 of sum_l |x_il m_lj|.
+// These differ where columns of the block differ in size and the matrix makes up for it. V is such a block (a
+// column whose Cholesky factor is 10^-6 of the others'), so is R at the set-up with a graded U, and A P, where a
+// smooth column of P has eigenvalues far below the others': there column l enters as 2^o V_l, and row l of the
+// matrix as 2^-o of it, with o from the norms of the columns. The k x k steps know them: zeta has the column norms of V,
+// Sigma those of R, and P^T A P = W^T (A P) is A P projected on the orthonormal W (emulated, Poisson 183^2, one smooth
+// column and three rough ones: (A P) T off by 7e-14 of its norm without and 5e-17 with them, FP64 sums 9e-17).
+// P has none: its columns are W's, of norm 1, and what CG adds to them.
 //
 // Widths. The row products see the block as rows of KV = max(KP, 8) columns and a Gram as rows of 16: for
 // a narrower block several rows make one, with the k x k matrix repeated on the diagonal (the diagonal
@@ -62,11 +70,11 @@ constexpr int kMxThreads = 256;  // threads per CTA
 constexpr int kMxGramBits = 56;  // B of the Grams
 constexpr unsigned kMxAll = 0xffffffffu;
 constexpr int kMxTiny = 192;    // a group with a scale exponent below this one counts as zero
-constexpr int kMxNaN = 0x4000;  // scale exponent of a column of a Gram that is not finite
+constexpr int kMxNaN = 0x4000;  // scale exponent of a group that is not finite
 
 __device__ __forceinline__ int mx_exponent(double x) { return (__double2hiint(x) >> 20) & 0x7FF; }
 
-// X of 2^o x (0 <= o < 128) in a group of scale exponent E (>= its own), to nearest (halves away from zero).
+// X of 2^o x (-128 < o < 128) in a group of scale exponent E (>= its own), to nearest (halves away from zero).
 template <int B>
 __device__ __forceinline__ long long mx_int(double x, int E, int o = 0) {
   const int h = __double2hiint(x), e = (h >> 20) & 0x7FF;
@@ -182,16 +190,44 @@ constexpr unsigned long long kMxStartSum =
     (unsigned long long)(kMxStart >> 8) + (unsigned long long)kMxStart * (1ull + 256ull + 65536ull + 16777216ull) +
     ((unsigned long long)(uint32_t)(kMxStart + (kMxStart << 8)) << 32);
 
-// Fills M from src(l, j) (KP x KP; all threads; the caller synchronises before and after).
+// Exponents o[l] (0 to 63) that bring columns l of a block to like size, from a k x k matrix src(j, l) whose
+// columns have the norms of the block's: the largest column has 0 (all threads; the caller synchronises before
+// and after).
 template <int KP, typename F>
-__device__ void mx_load_matrix(F src, MxMatrix<KP>& M) {
-  using W = MxRows<KP>;
+__device__ void mx_column_exponents(F src, int (&o)[KP]) {
+  __shared__ int c[KP];
   const int tid = threadIdx.x;
   if (tid < KP) {
     int e = 0;
 #pragma unroll 8
-    for (int l = 0; l < KP; ++l) e = max(e, mx_exponent(src(l, tid)));
-    M.e[tid] = e;
+    for (int j = 0; j < KP; ++j) e = max(e, mx_exponent(src(j, tid)));
+    c[tid] = e;
+  }
+  __syncthreads();
+  if (tid < KP) {
+    int m = 0;
+#pragma unroll 8
+    for (int j = 0; j < KP; ++j) m = max(m, c[j]);
+    o[tid] = min(m - c[tid], 63);
+  }
+}
+
+// Fills M from src(l, j) (KP x KP; all threads; the caller synchronises before and after). o: row l enters as
+// 2^-o[l] src(l, j), for blocks whose columns enter as 2^o[l] of theirs; or NULL.
+template <int KP, typename F>
+__device__ void mx_load_matrix(F src, const int* o, MxMatrix<KP>& M) {
+  using W = MxRows<KP>;
+  const int tid = threadIdx.x;
+  if (tid < KP) {
+    int e = 0;
+    bool bad = false;
+#pragma unroll 8
+    for (int l = 0; l < KP; ++l) {
+      const int x = mx_exponent(src(l, tid));
+      bad |= x == 0x7FF;
+      e = max(e, x - (o != nullptr ? o[l] : 0));
+    }
+    M.e[tid] = bad ? kMxNaN : e;
   }
   __syncthreads();
   for (int q = tid; q < W::KS * W::NB * 32; q += kMxThreads) {
@@ -199,7 +235,9 @@ __device__ void mx_load_matrix(F src, MxMatrix<KP>& M) {
     const int n = 8 * nb + (lane >> 2), k0 = 16 * ks + 2 * (lane & 3);
     // view matrix: KP x KP blocks on the diagonal
     auto at = [&](int k) {
-      return (k < W::KV && k / KP == n / KP) ? mx_int<W::B>(src(k % KP, n % KP), M.e[n % KP]) : 0LL;
+      return (k < W::KV && k / KP == n / KP)
+                 ? mx_int<W::B>(src(k % KP, n % KP), M.e[n % KP], o != nullptr ? -o[k % KP] : 0)
+                 : 0LL;
     };
     uint32_t d0[kMxDigits], d1[kMxDigits];
     mx_digits(at(k0), at(k0 + 1), d0);
@@ -216,21 +254,41 @@ struct MxTile {
   uint32_t a[kMxDigits][2 * W::NB];
   int e[2];
 
-  // v[c][r]: columns 8 c + 2 t, + 1 of view row g + 8 r
-  __device__ __forceinline__ void split(const double2 (&v)[W::NB][2]) {
+  // the largest over the lanes of a row: at KP = 4 lanes t = 0, 1 hold one row of the block and t = 2, 3 the
+  // next one, here and in the results
+  static __device__ __forceinline__ int row_max(int m) {
+    m = max(m, __shfl_xor_sync(kMxAll, m, 1));
+    if constexpr (KP >= 8) m = max(m, __shfl_xor_sync(kMxAll, m, 2));
+    return m;
+  }
+
+  // v[c][r]: columns 8 c + 2 t, + 1 of view row g + 8 r. o: column j enters as 2^o[j] of it; or NULL.
+  __device__ __forceinline__ void split(const double2 (&v)[W::NB][2], const int* o) {
+    int ox[W::NB], oy[W::NB];
+#pragma unroll
+    for (int c = 0; c < W::NB; ++c) {
+      const int j = (8 * c + 2 * (threadIdx.x & 3)) % KP;
+      ox[c] = o != nullptr ? o[j] : 0;
+      oy[c] = o != nullptr ? o[j + 1] : 0;
+    }
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
       int m = 0;
 #pragma unroll
-      for (int c = 0; c < W::NB; ++c) m = max(m, max(mx_exponent(v[c][r].x), mx_exponent(v[c][r].y)));
-      m = max(m, __shfl_xor_sync(kMxAll, m, 1));
-      // at KP = 4 lanes t = 0, 1 hold one row of the block and t = 2, 3 the next one, here and in the results
-      if constexpr (KP >= 8) m = max(m, __shfl_xor_sync(kMxAll, m, 2));
+      for (int c = 0; c < W::NB; ++c)
+        m = max(m, max(mx_exponent(v[c][r].x) + ox[c], mx_exponent(v[c][r].y) + oy[c]));
+      m = row_max(m);
+      if (__any_sync(kMxAll, m >= 0x7FF)) {  // an infinity or a NaN, or large values of a column that o raises
+        int raw = 0;
+#pragma unroll
+        for (int c = 0; c < W::NB; ++c) raw = max(raw, max(mx_exponent(v[c][r].x), mx_exponent(v[c][r].y)));
+        if (row_max(raw) == 0x7FF) m = kMxNaN;
+      }
       e[r] = m;
 #pragma unroll
       for (int c = 0; c < W::NB; ++c) {
         uint32_t d[kMxDigits];
-        mx_digits(mx_int<W::B>(v[c][r].x, e[r]), mx_int<W::B>(v[c][r].y, e[r]), d);
+        mx_digits(mx_int<W::B>(v[c][r].x, e[r], ox[c]), mx_int<W::B>(v[c][r].y, e[r], oy[c]), d);
 #pragma unroll
         for (int t = 0; t < kMxDigits; ++t) a[t][2 * c + r] = d[t];
       }
@@ -266,7 +324,7 @@ struct MxTile {
     for (int q = 0; q < 4; ++q) {
       const int f = M.e[j + (q & 1)], er = e[q >> 1];
       v[q] = mx_double((long long)sum[q], er + f - 2044 - 2 * W::B + 56);
-      if (max(f, er) == 0x7FF) v[q] = mx_nan();
+      if (max(f, er) == kMxNaN) v[q] = mx_nan();
     }
     y[0] = make_double2(v[0], v[1]);
     y[1] = make_double2(v[2], v[3]);
@@ -300,20 +358,25 @@ __device__ __forceinline__ void mx_store_rows(double* X, size_t row, size_t nf, 
 }
 
 // Block update of Algorithm 1 (as k_axpy): X~ += P T, R -= (A P) T, V = W - (A P) Xi, and the CTA partials
-// of nu at part[NPACK + j]. RFREE: R is neither read nor written, and there are no norms. Tiles of 16
+// of nu at part[NPACK + j]. Gp: the upper triangle of P^T (A P). RFREE: R is neither read nor written, and there are no norms. Tiles of 16
 // view rows are dealt to the warps of the grid in turn (their sums do not depend on the order).
 template <int KP, bool RFREE>
 __global__ void __launch_bounds__(kMxThreads, KP >= 32 ? 1 : 2)
 k_axpy_mx(int n, const double* __restrict__ P, const double* __restrict__ Q, const double* __restrict__ W,
           double* __restrict__ R, double* __restrict__ Xt, double* __restrict__ V, const double* __restrict__ Tg,
-          const double* __restrict__ Xig, const double* __restrict__ wdiag, double* __restrict__ part, int pstride,
-          const SolveState* __restrict__ st) {
+          const double* __restrict__ Xig, const double* __restrict__ Gp, const double* __restrict__ wdiag,
+          double* __restrict__ part, int pstride, const SolveState* __restrict__ st) {
   using M = MxRows<KP>;
   if (st->done) return;
-  __shared__ MxMatrix<KP> T, Xi;
+  __shared__ MxMatrix<KP> T, Xi;                                               // of P, of A P
+  __shared__ typename std::conditional<RFREE, int, MxMatrix<KP>>::type Tq;     // T for A P
   __shared__ double red[RFREE ? 1 : kMxThreads / 32][KP];
-  mx_load_matrix<KP>([&](int l, int j) { return __ldg(Tg + l + j * KP); }, T);
-  mx_load_matrix<KP>([&](int l, int j) { return __ldg(Xig + l + j * KP); }, Xi);
+  __shared__ int oq[KP];
+  auto tg = [&](int l, int j) { return __ldg(Tg + l + j * KP); };
+  mx_column_exponents<KP>([&](int j, int l) { return __ldg(Gp + pidx(min(j, l), max(j, l))); }, oq);
+  mx_load_matrix<KP>(tg, nullptr, T);  // (its barrier stands before the first use of oq)
+  mx_load_matrix<KP>([&](int l, int j) { return __ldg(Xig + l + j * KP); }, oq, Xi);
+  if constexpr (!RFREE) mx_load_matrix<KP>(tg, oq, Tq);
   __syncthreads();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
   const size_t nf = (size_t)n * KP, nv = (nf + M::KV - 1) / M::KV;
@@ -327,7 +390,7 @@ k_axpy_mx(int n, const double* __restrict__ P, const double* __restrict__ Q, con
     double2 v[M::NB][2], x[M::NB][2], y[2];
     mx_load_rows<KP>(P, row, nf, t, v);
     mx_load_rows<KP>(Xt, row, nf, t, x);
-    tile.split(v);
+    tile.split(v, nullptr);
     mx_load_rows<KP>(Q, row, nf, t, v);
 #pragma unroll
     for (int c = 0; c < M::NB; ++c) {
@@ -340,7 +403,7 @@ k_axpy_mx(int n, const double* __restrict__ P, const double* __restrict__ Q, con
     }
     mx_store_rows<KP>(Xt, row, nf, t, x);
     mx_load_rows<KP>(W, row, nf, t, x);
-    tile.split(v);
+    tile.split(v, oq);
     if constexpr (!RFREE) mx_load_rows<KP>(R, row, nf, t, v);
 #pragma unroll
     for (int c = 0; c < M::NB; ++c) {
@@ -355,7 +418,7 @@ k_axpy_mx(int n, const double* __restrict__ P, const double* __restrict__ Q, con
     if constexpr (!RFREE) {
 #pragma unroll
       for (int c = 0; c < M::NB; ++c) {
-        tile.times(T, c, y);
+        tile.times(Tq, c, y);
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
           v[c][r].x -= y[r].x;
@@ -401,7 +464,8 @@ k_axpy_mx(int n, const double* __restrict__ P, const double* __restrict__ Q, con
   }
 }
 
-// W/P update of Algorithm 1 (as k_pw): W = V zeta^{-1}, P = W + P zeta^T (SETP: P = W).
+// W/P update of Algorithm 1 (as k_pw): W = V zeta^{-1}, P = W + P zeta^T (SETP: P = W; Zg is then Sigma, V is R).
+// V = Q zeta with orthonormal Q, so that the columns of zeta have the norms of V's.
 template <int KP, bool SETP>
 __global__ void __launch_bounds__(kMxThreads, KP >= 32 ? 1 : 2)
 k_pw_mx(int n, const double* __restrict__ V, double* __restrict__ W, double* __restrict__ P,
@@ -410,8 +474,11 @@ k_pw_mx(int n, const double* __restrict__ V, double* __restrict__ W, double* __r
   if (st != nullptr && st->pw_skip) return;
   __shared__ MxMatrix<KP> Zi;
   __shared__ typename std::conditional<SETP, int, MxMatrix<KP>>::type Zt;
-  mx_load_matrix<KP>([&](int l, int j) { return __ldg(Zinvg + l + j * KP); }, Zi);
-  if constexpr (!SETP) mx_load_matrix<KP>([&](int l, int j) { return __ldg(Zg + j + l * KP); }, Zt);
+  __shared__ int ov[KP];
+  mx_column_exponents<KP>([&](int j, int l) { return __ldg(Zg + j + l * KP); }, ov);
+  __syncthreads();
+  mx_load_matrix<KP>([&](int l, int j) { return __ldg(Zinvg + l + j * KP); }, ov, Zi);
+  if constexpr (!SETP) mx_load_matrix<KP>([&](int l, int j) { return __ldg(Zg + j + l * KP); }, nullptr, Zt);
   __syncthreads();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
   const size_t nf = (size_t)n * KP, nv = (nf + M::KV - 1) / M::KV;
@@ -421,13 +488,13 @@ k_pw_mx(int n, const double* __restrict__ V, double* __restrict__ W, double* __r
     MxTile<KP> tile;
     double2 v[M::NB][2], w[M::NB][2], y[2];
     mx_load_rows<KP>(V, row, nf, t, v);
-    tile.split(v);
+    tile.split(v, ov);
     if constexpr (!SETP) mx_load_rows<KP>(P, row, nf, t, v);
 #pragma unroll
     for (int c = 0; c < M::NB; ++c) tile.times(Zi, c, w[c]);
     mx_store_rows<KP>(W, row, nf, t, w);
     if constexpr (!SETP) {
-      tile.split(v);
+      tile.split(v, nullptr);
 #pragma unroll
       for (int c = 0; c < M::NB; ++c) {
         tile.times(Zt, c, y);

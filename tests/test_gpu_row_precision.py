@@ -134,3 +134,53 @@ def test_product_gram_of_rows_in_different_units(mb, s):
     cond = np.linalg.cond(G.astype(np.float64))
     assert cond < 4
     assert np.abs(T - ref).max() <= (30 + 8 * s) * U53 * cond * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("s", [4, 8, 13, 32])
+def test_columns_of_different_size(mb, s):
+    """First residuals from 10^-5 to 1 of b (U_j solves A U_j = b - r_j; the last one is stretched so that the
+    set-up's common factor of U, sqrt(s) |b| / |A U|, is 1): W = R Sigma^-1 column by column within 2^-53 in the root
+    mean square (an FP64 product with a graded Sigma^-1 is a rounding and little more)."""
+    scipy_linalg = pytest.importorskip("scipy.sparse.linalg")
+    A = wl.poisson2d(183)
+    r = wl.initial_block(A.n, s, 1) * 10.0 ** (np.arange(s) * 5.0 / (s - 1) - 5.0)
+    b = wl.rhs(A.n, 0)
+    AU = b[:, None] - r
+    AU[:, -1] *= np.sqrt((s * (b ** 2).sum() - (AU[:, :-1] ** 2).sum()) / (AU[:, -1] ** 2).sum())
+    U = np.asfortranarray(scipy_linalg.splu(A.to_scipy().tocsc()).solve(AU))
+    (z,) = states(mb, A, b, U, s, 0, (0,))
+    size = np.sqrt((z["R"] ** 2).sum(0))
+    assert size.max() > 1e4 * size.min()  # the columns do differ
+    W = z["W"].astype(LD)
+    E = product(z["R"], fit(z["R"], W)) - W
+    assert (np.sqrt((E ** 2).sum(0) / (W ** 2).sum(0)) <= U53).all()
+
+
+@pytest.mark.parametrize("s", [4, 11, 32])
+def test_smooth_column_beside_rough_ones(mb, s):
+    """The first residual is smooth, the others are not: the first column of A P is 10^3 to 10^4 below the others, and
+    Xi makes up for it. R = R_0 - (A P) T column by column: every one of s FMAs rounds to 2^-53 of a partial sum, which
+    is at most |R_0| + sum_l |(A P)_l| |T_lj|."""
+    A = wl.poisson2d(183)
+    n = A.n
+    x = np.sin(np.pi * np.arange(1, 184) / 184)
+    smooth = np.outer(x, x).ravel()
+    b = smooth + 1e-5 * wl.rhs(n, 0)
+    U = wl.initial_block(n, s, 1)
+    U[:, 0] = -100.0 * smooth
+    z, one = states(mb, A, b, U, s, 0, (0, 1))
+    P = torch.zeros((n, mb.mbpcg_k_padded_width(s)), dtype=torch.float64, device="cuda")
+    P[:, :s] = torch.as_tensor(z["P"], device="cuda")
+    sv = mb.Solver(A, s=s)
+    try:
+        Q = sv.apply(P)[:, :s].cpu().numpy()  # the loop's A P, bit for bit
+    finally:
+        sv.close()
+    size = np.sqrt((Q ** 2).sum(0))
+    assert size.max() > 1e3 * size[0]
+    D = z["R"].astype(LD) - one["R"]
+    T = fit(Q, D)
+    E = product(Q, T) - D
+    bound = np.sqrt((z["R"] ** 2).sum(0)) + (size[:, None] * np.abs(T)).sum(0)
+    err = np.sqrt((E ** 2).sum(0)) / bound
+    assert (err <= s * U53).all(), err / U53
