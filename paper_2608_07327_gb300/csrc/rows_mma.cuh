@@ -51,7 +51,7 @@
 // blocks of the Gram summed). Every row of the block keeps a scale of its own: neighbouring unknowns may be in
 // different units, and a row 10^6 below its neighbour would lose 20 bits to a common one.
 //
-// A group that holds an infinity or a NaN has E = 0x7FF, and what is formed from it is NaN. A group below
+// A group that holds an infinity or a NaN has E = kMxNaN, and what is formed from it is NaN. A group below
 // 2^-831 counts as zero (the solver squares norms: it can use nothing below 2^-511).
 #pragma once
 #include <cuda_fp16.h>
@@ -271,20 +271,26 @@ struct MxTile {
       ox[c] = o != nullptr ? o[j] : 0;
       oy[c] = o != nullptr ? o[j + 1] : 0;
     }
-#pragma unroll
-    for (int r = 0; r < 2; ++r) {
+    auto largest = [&](int r, bool raw) {
       int m = 0;
 #pragma unroll
       for (int c = 0; c < W::NB; ++c)
-        m = max(m, max(mx_exponent(v[c][r].x) + ox[c], mx_exponent(v[c][r].y) + oy[c]));
-      m = row_max(m);
-      if (__any_sync(kMxAll, m >= 0x7FF)) {  // an infinity or a NaN, or large values of a column that o raises
-        int raw = 0;
+        m = max(m, max(mx_exponent(v[c][r].x) + (raw ? 0 : ox[c]), mx_exponent(v[c][r].y) + (raw ? 0 : oy[c])));
+      return row_max(m);
+    };
+    e[0] = largest(0, false);
+    e[1] = largest(1, false);
+    if (o == nullptr) {
 #pragma unroll
-        for (int c = 0; c < W::NB; ++c) raw = max(raw, max(mx_exponent(v[c][r].x), mx_exponent(v[c][r].y)));
-        if (row_max(raw) == 0x7FF) m = kMxNaN;
-      }
-      e[r] = m;
+      for (int r = 0; r < 2; ++r)
+        if (e[r] == 0x7FF) e[r] = kMxNaN;
+    } else if (__any_sync(kMxAll, max(e[0], e[1]) >= 0x7FF)) {  // not finite, or large values of a column that o raises
+#pragma unroll
+      for (int r = 0; r < 2; ++r)
+        if (largest(r, true) == 0x7FF) e[r] = kMxNaN;
+    }
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
 #pragma unroll
       for (int c = 0; c < W::NB; ++c) {
         uint32_t d[kMxDigits];
@@ -292,7 +298,6 @@ struct MxTile {
 #pragma unroll
         for (int t = 0; t < kMxDigits; ++t) a[t][2 * c + r] = d[t];
       }
-    }
   }
 
   // Columns 8 nb + 2 t, + 1 of the two rows times M: y[r].

@@ -184,3 +184,19 @@ def test_smooth_column_beside_rough_ones(mb, s):
     bound = np.sqrt((z["R"] ** 2).sum(0)) + (size[:, None] * np.abs(T)).sum(0)
     err = np.sqrt((E ** 2).sum(0)) / bound
     assert (err <= s * U53).all(), err / U53
+
+
+@pytest.mark.parametrize("s", [4, 8, 16, 32])
+@pytest.mark.parametrize("value", [np.nan, -np.inf])
+def test_non_finite_initial_block_breaks_down_at_the_set_up(mb, s, value):
+    """One value of U that is not finite makes the first residual's Gram matrix NaN: its Cholesky factor has no
+    positive pivot, and no iteration is made."""
+    A = wl.poisson2d(183)
+    b, U = wl.rhs(A.n, 0), wl.initial_block(A.n, s, 1)
+    U[20000, s - 1] = value
+    sv = mb.Solver(A, s=s)
+    try:
+        _, info = sv.solve(b, U, tol=1e-8)
+    finally:
+        sv.close()
+    assert (info["status"], info["iterations"]) == (mb.MBPCG_BREAKDOWN, 0)
