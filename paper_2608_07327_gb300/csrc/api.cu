@@ -927,14 +927,18 @@ cudaError_t capture_solve(mbpcg_ctx* h, cudaGraph_t g, cudaGraphConditionalHandl
         // this GPU, on top of ~1 us per kernel; every loop kernel returns at once after the
         // iteration in which the solve stopped, and the last one of a pass sets the condition
         h->use_cond = 1;
+        const cudaError_t pending = cudaPeekAtLastError();  // not of this call
         for (int u = 0; u < (in_loop_cluster(h) ? 1 : kBodyUnroll); ++u) {
           if (cg) enqueue_cg_body(h);
           else if (h->dm.mixed) enqueue_mbpcg_body_f(h);
           else enqueue_mbpcg_body(h);
         }
         h->use_cond = 0;
+        // a launch that was refused is not in the graph, and a body without it might never clear the condition
+        const cudaError_t refused = pending == cudaSuccess ? cudaGetLastError() : cudaSuccess;
         cudaGraph_t b2 = nullptr;
         e = cudaStreamEndCapture(h->stream, &b2);
+        if (e == cudaSuccess) e = refused;
       }
     }
   }

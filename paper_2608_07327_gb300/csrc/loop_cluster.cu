@@ -715,7 +715,7 @@ int loop_cluster_ready(int kp, int n, int slice) {
              cudaSuccess &&
          cudaOccupancyMaxActiveClusters(&clusters, k, &c) == cudaSuccess;
   }
-  cudaGetLastError();  // a refusal here only means the launches of the row kernels
+  if (!ok) cudaGetLastError();  // a refusal here only means the launches of the row kernels
   return ok && clusters > 0 && 2 * (long long)zcap >= slice ? zcap : -1;
 }
 
@@ -723,8 +723,9 @@ void launch_loop_cluster(cudaStream_t s, int kp, const LoopArgs& a, int iters, c
                          int use_cond) {
   cudaLaunchAttribute at;
   const cudaLaunchConfig_t c = lc_config(kp, a.n, a.zcap, s, &at);
-  cudaLaunchKernelEx(&c, lc_kernel(kp), a.n, a.rp, a.ci, a.av, a.X, a.R, a.W, a.P, a.wdiag, a.Sigma,
-                     a.st, a.zcap, iters, cond, use_cond);
+  // (a launch that is refused is the thread's last error, as with the other kernels)
+  (void)cudaLaunchKernelEx(&c, lc_kernel(kp), a.n, a.rp, a.ci, a.av, a.X, a.R, a.W, a.P, a.wdiag, a.Sigma, a.st,
+                           a.zcap, iters, cond, use_cond);
 }
 
 }  // namespace mbpcg
