@@ -234,8 +234,8 @@ struct LoopArgs {
 };
 bool loop_cluster_fits(int kp, int n, long long nnz);  // the sizes it is for
 void loop_cluster_slice(cudaStream_t s, int n, const int* rp, int* out);
-// -1 unless the blocks fit in shared memory and the device can schedule the cluster; slice: entries of A in
-// the largest of the CTAs' row ranges (loop_cluster_slice)
+// -1 unless the blocks fit in shared memory, no CTA has far more of A than the others and the device can schedule
+// the cluster; slice: entries of A in the largest of the CTAs' row ranges (loop_cluster_slice)
 int loop_cluster_ready(int kp, int n, int slice);
 void launch_loop_cluster(cudaStream_t s, int kp, const LoopArgs& a, int iters, cudaGraphConditionalHandle cond,
                          int use_cond);

@@ -692,11 +692,15 @@ cudaLaunchConfig_t lc_config(int kp, int n, int zcap, cudaStream_t s, cudaLaunch
 //   (1.35 M) 33.7 / 32.1, 4096 (1.83 M) 33.7 / 38.6; 27-point, s = 4: n = 1728 38.6 / 13.9, 5832 (1.21 M) 36.9 /
 //   29.6; s = 8: 1728 (1.04 M) 37.9 / 28.7, 2197 (1.33 M) 37.7 / 34.7.
 // From KP = 16 the k x k steps are larger than one warp's work (clusters of their own, small_warp.cu).
-bool loop_cluster_fits(int kp, int n, long long nnz) {
-  if (kp > 8) return false;
-  const long long row = (long long)kp * (2 * (kp / 2 + 1) + 5 * kp + 1);
-  return nnz * kp + n * row <= 1400000;
+static long long lc_fmas(int kp, int n, long long nnz) {
+  return nnz * kp + n * ((long long)kp * (2 * (kp / 2 + 1) + 5 * kp + 1));
 }
+bool loop_cluster_fits(int kp, int n, long long nnz) { return kp <= 8 && lc_fmas(kp, n, nnz) <= 1400000; }
+
+// The same for the CTA with the most entries: where a few neighbouring rows have most of A, one SM does their
+// part of the product. us per iteration, row kernels / this kernel, at 16 times the FMAs of that CTA: s = 8, n =
+// 1500: 2.25 M 64 / 61, 3.13 M 77 / 95, 3.88 M 88 / 143; s = 4, n = 2000: 2.08 M 108 / 82.
+static bool lc_balanced(int kp, int n, int slice) { return lc_fmas(kp, n, 16LL * slice) <= 2250000; }
 
 void loop_cluster_slice(cudaStream_t s, int n, const int* rp, int* out) { k_lc_slice<<<1, 32, 0, s>>>(n, rp, out); }
 
@@ -706,6 +710,7 @@ int loop_cluster_ready(int kp, int n, int slice) {
   cudaFuncAttributes fa;
   cudaLaunchAttribute at;
   int clusters = 0, zcap = -1;
+  if (!lc_balanced(kp, n, slice)) return -1;
   bool ok = cudaFuncGetAttributes(&fa, k) == cudaSuccess && lc_smem(kp, n, 0) + fa.sharedSizeBytes <= kSmem;
   if (ok) {
     zcap = (int)std::min((size_t)slice, (kSmem - fa.sharedSizeBytes - lc_smem(kp, n, 0)) / 12);

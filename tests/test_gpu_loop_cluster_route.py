@@ -1,0 +1,67 @@
+"""Which systems iterate in one thread-block cluster, read from the kernels that a solve launches (launch mode EAGER, in
+which a profiler sees them), and the entries of A that its shared memory does not hold."""
+import numpy as np
+import pytest
+
+import workloads as wl
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def mb():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2608_07327_gb300 as mb
+    mb.lib()
+    with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]):  # the first one sees no kernels
+        torch.zeros(10, device="cuda").add_(1)
+        torch.cuda.synchronize()
+    return mb
+
+
+def kernels(mb, A, s, **options):
+    """Names of the kernels of three iterations."""
+    sv = mb.Solver(A, s=s, launch_mode=mb.MBPCG_LAUNCH_EAGER, **options)
+    b, U = wl.rhs(A.n, 0), wl.initial_block(A.n, s, 1)
+    try:
+        sv.solve(b, U, tol=1e-14, maxit=3)
+        with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
+            sv.solve(b, U, tol=1e-14, maxit=3)
+            torch.cuda.synchronize()
+    finally:
+        sv.close()
+    return {e.name for e in prof.events() if e.device_type == torch.autograd.DeviceType.CUDA}
+
+
+def in_cluster(names):
+    assert any("k_small_true" in k for k in names)  # the profiler sees the library's kernels
+    return any("k_loop_cluster" in k for k in names)
+
+
+def crowded(n, rows, width):
+    """The first rows have most of the entries."""
+    rng = np.random.default_rng(3)
+    D = np.zeros((n, n))
+    for i in range(rows):
+        c = rng.choice(n, width, replace=False)
+        D[i, c] = D[c, i] = -1e-3 * rng.random(width)
+    np.fill_diagonal(D, rng.uniform(2.0, 3.0, n))
+    r, c = np.nonzero(D)
+    rp = np.zeros(n + 1, np.int32)
+    np.cumsum(np.bincount(r, minlength=n), out=rp[1:])
+    return wl.CSR(n, rp, c.astype(np.int32), D[r, c])
+
+
+@pytest.mark.parametrize("name,factory,s,options,expected", [
+    ("poisson64_s4", lambda: wl.poisson2d(64), 4, {}, True),
+    ("poisson55_s8", lambda: wl.poisson2d(55), 8, {}, True),
+    ("poisson60_s8_too_large", lambda: wl.poisson2d(60), 8, {}, False),
+    ("poisson30_s9", lambda: wl.poisson2d(30), 9, {}, False),
+    ("poisson30_s4_implicit", lambda: wl.poisson2d(30), 4, {"residual_mode": 1}, False),
+    ("crowded_s8", lambda: crowded(1500, 94, 100), 8, {}, True),
+    ("crowded_s8_one_sm_has_most", lambda: crowded(1500, 94, 260), 8, {}, False),
+])
+def test_route(mb, name, factory, s, options, expected):
+    assert in_cluster(kernels(mb, factory(), s, **options)) is expected
