@@ -65,3 +65,33 @@ def crowded(n, rows, width):
 ])
 def test_route(mb, name, factory, s, options, expected):
     assert in_cluster(kernels(mb, factory(), s, **options)) is expected
+
+
+# 16 CTAs with some 14,600 (27-point) and 10,000 entries of A in shared memory each
+@pytest.mark.parametrize("name,factory,precond", [
+    ("stencil25", lambda: wl.stencil27(25, 5), 0),
+    ("stencil24_jacobi", lambda: wl.stencil27(24, 6), 1),
+    ("poisson181", lambda: wl.poisson2d(181), 0),
+])
+def test_entries_past_shared_memory(mb, orc, name, factory, precond):
+    """Rows whose entries come from global memory, and the row at the limit. Sums of n <= 33,000 terms in another
+    order than the oracle's, n x 2^-53 at worst, times what the first steps magnify (below 10): 5e-11."""
+    A = factory()
+    rows = [A.n * k // 16 for k in range(17)]
+    most = max(A.row_ptr[rows[k + 1]] - A.row_ptr[rows[k]] for k in range(16))
+    blocks = 6 * 8 * -(-A.n // 16)
+    assert 12 * most + blocks > 227 * 1024 - 4 * -(-A.n // 16) - 8192  # more than fits (8 KB: the kernel's own)
+    assert in_cluster(kernels(mb, A, 1, precond=precond))
+    b, U = wl.rhs(A.n, 0), wl.initial_block(A.n, 1, 1)
+    sv = mb.Solver(A, s=1, precond=precond)
+    try:
+        for m in (1, 3):
+            got, st = sv.run_iterations(b, U, m)
+            ref, st_o = orc.mbpcg_state(A, b, U, m, precond=precond)
+            assert st == st_o
+            for key in ("X0", "Xt", "R", "W", "P", "Sigma"):
+                assert np.abs(got[key] - ref[key]).max() <= 5e-11 * np.abs(ref[key]).max(), (key, m)
+        x, info = sv.solve(b, U, tol=1e-8)
+    finally:
+        sv.close()
+    assert info["status"] == 0 and np.linalg.norm(b - A.to_scipy() @ x) <= 1e-8 * np.linalg.norm(b)
