@@ -115,10 +115,10 @@ Dims make_dims(int n, long long nnz, int s, int algo, int dense, int sms) {
 //     diffusion 24^3, kp = 32 (2^18.8): 22 against 24; kp = 16 (2^17.8): 15 against 10.6).
 void apply_mx(Dims& d) {
   const long long values = (long long)d.n * d.kp;
-  if (d.dense || d.algo != MBPCG_ALGO_MBPCG || d.kp < 4 || values < (1LL << 17)) return;
+  if (d.dense || d.algo != MBPCG_ALGO_MBPCG || d.kp < kMxMinKP || values < (1LL << 17)) return;
   d.mx = 1;
-  d.mx_pw = d.kp >= 8;
-  d.mx_gram = d.kp >= 16 && values >= (1LL << 19);
+  d.mx_pw = d.kp >= kMxPwMinKP;
+  d.mx_gram = d.kp >= kMxProductMinKP && values >= (1LL << 19);
   const long long view = (values + 15) / 16, want = (view + 127) / 128;
   d.nb_mx = (int)(want < 2LL * d.sms ? want : 2LL * d.sms);
   if (d.nb_mx > d.nbmax) d.nbmax = d.nb_mx;
@@ -679,11 +679,11 @@ void enqueue_product(mbpcg_ctx* h, const RowOps* ops, const double* X, double* Y
   } else if (h->prod64 == MBPCG_PRODUCT_CSR_TILED) {
     spmm_tiled(h->stream, dm.kp, dm.nb, dm.n, h->rp, h->av, h->plan, X, Y, h->part, dm.pstride, st,
                gram && !dm.mx_gram);
-    if (gram && dm.mx_gram) ops->gram_mx(h->stream, dm.nb_mx, dm.n, X, Y, nullptr, bal, h->part, dm.pstride, st);
+    if (gram && dm.mx_gram) ops->product_gram_mx(h->stream, dm.nb_mx, dm.n, X, Y, bal, h->part, dm.pstride, st);
   } else {
     ops->spmm(h->stream, dm.nb, dm.n, h->rp, h->ci, h->av, X, Y, h->part, dm.pstride, st,
               gram && !dm.mx_gram ? (spmm_by_tiles(dm) ? 2 : 1) : 0);
-    if (gram && dm.mx_gram) ops->gram_mx(h->stream, dm.nb_mx, dm.n, X, Y, nullptr, bal, h->part, dm.pstride, st);
+    if (gram && dm.mx_gram) ops->product_gram_mx(h->stream, dm.nb_mx, dm.n, X, Y, bal, h->part, dm.pstride, st);
   }
 }
 
@@ -713,7 +713,7 @@ void enqueue_mbpcg_setup(mbpcg_ctx* h) {
   enqueue_reduce(h, 3, nullptr);
   k_small_setup<<<1, 1, 0, h->stream>>>(h->st, h->red);
   ops->init(h->stream, dm.nb, n, h->s, h->U, h->Q, h->bs, h->X0, h->Xt, h->R, h->part, dm.pstride, h->st, !dm.mx);
-  if (dm.mx) ops->gram_mx(h->stream, dm.nb_mx, n, h->R, h->R, nullptr, nullptr, h->part, dm.pstride, nullptr);
+  if (dm.mx) ops->gram_mx(h->stream, dm.nb_mx, n, h->R, nullptr, nullptr, h->part, dm.pstride, nullptr);
   enqueue_reduce(h, npack(kp), nullptr, dm.mx);
   launch_small_sigma(h->stream, kp, h->st, h->red, h->Sigma, h->SigmaInv);
   if (dm.mx_pw) ops->pw_mx(h->stream, dm.nb_mx, n, h->R, h->W, h->P, h->SigmaInv, h->Sigma, nullptr, 1);
@@ -747,9 +747,9 @@ void enqueue_mbpcg_body(mbpcg_ctx* h) {
   } else if (dm.mx) {
     ops->axpy_mx(h->stream, dm.nb_mx, n, h->P, h->Q, h->W, h->R, h->Xt, h->V, h->T, h->Xi, h->red, h->wdiag, h->part,
                  dm.pstride, h->st, h->rfree);
-    ops->gram_mx(h->stream, dm.nb_mx, n, h->V, h->V, nullptr, nullptr, h->part, dm.pstride, h->st);
+    ops->gram_mx(h->stream, dm.nb_mx, n, h->V, nullptr, nullptr, h->part, dm.pstride, h->st);
     if (h->rfree && h->wdiag != nullptr)  // V^T D^2 V
-      ops->gram_mx(h->stream, dm.nb_mx, n, h->V, h->V, h->sqd, h->wdiag, h->part + npack(kp) + kp, dm.pstride,
+      ops->gram_mx(h->stream, dm.nb_mx, n, h->V, h->sqd, h->wdiag, h->part + npack(kp) + kp, dm.pstride,
                    h->st);
   } else {
     ops->axpy(h->stream, dm.nb, n, h->P, h->Q, h->W, h->R, h->Xt, h->V, h->T, h->Xi, h->wdiag, h->part, dm.pstride,
@@ -781,7 +781,7 @@ void enqueue_mbpcg_exit(mbpcg_ctx* h) {
   if (h->rfree) ops->rsig(h->stream, dm.nb, n, h->V, h->W, h->Sigma, h->R, h->st);
   ops->ls_gram(h->stream, dm.nb, n, h->R, h->rhs, h->sqd, h->part, dm.pstride, !dm.mx);
   if (dm.mx) {  // (D R)^T (D R); the other entries from their own partials
-    ops->gram_mx(h->stream, dm.nb_mx, n, h->R, h->R, h->sqd, h->wdiag, h->part, dm.pstride, nullptr);
+    ops->gram_mx(h->stream, dm.nb_mx, n, h->R, h->sqd, h->wdiag, h->part, dm.pstride, nullptr);
     enqueue_reduce(h, npack(kp), nullptr, 1);
     enqueue_reduce(h, kp + 1, nullptr, 0, npack(kp));
   } else {

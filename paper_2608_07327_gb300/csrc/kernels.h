@@ -22,6 +22,10 @@ inline cudaError_t ensure_dynamic_smem(K* func, size_t bytes) {
 }
 
 
+// Narrowest blocks of the row passes on the tensor cores (rows_mma.cuh; the figures stand at apply_mx in api.cu):
+// block update and the Grams of one block, W/P update, Gram of the product.
+constexpr int kMxMinKP = 4, kMxPwMinKP = 8, kMxProductMinKP = 16;
+
 // Host launchers of the row kernels for one padded width KP (defined in inst_kp*.cu).
 struct RowOps {
   int kp;
@@ -59,11 +63,13 @@ struct RowOps {
                    const SolveState* st);
   void (*pw_pre)(cudaStream_t, int n, const double* VZi, const double* PZt, double* W, double* P, const SolveState* st,
                  int* emax);
-  // the row passes on the tensor cores (rows_mma.cuh; KP >= 4): the Gram X^T Y (Y = X: X^T D^2 X with
-  // D and D^2, or NULL; otherwise d2 is the diagonal that balances the rows, or NULL), the block update without its Gram (G: P^T A P, packed),
-  // the W/P update (setp: Z is the Cholesky factor Sigma of V)
-  void (*gram_mx)(cudaStream_t, int nb, int n, const double* X, const double* Y, const double* d, const double* d2,
-                  double* part, int pstride, const SolveState* st);
+  // the row passes on the tensor cores (NULL below their widths): the Gram X^T D^2 X (D and D^2, or NULL), the
+  // product's Gram P^T Q (diag: balances the rows, or NULL), the block update without its Gram (G: P^T A P,
+  // packed), the W/P update (setp: Z is the Cholesky factor Sigma of V)
+  void (*gram_mx)(cudaStream_t, int nb, int n, const double* X, const double* d, const double* d2, double* part,
+                  int pstride, const SolveState* st);
+  void (*product_gram_mx)(cudaStream_t, int nb, int n, const double* P, const double* Q, const double* diag,
+                          double* part, int pstride, const SolveState* st);
   void (*axpy_mx)(cudaStream_t, int nb, int n, const double* P, const double* Q, const double* W, double* R,
                   double* Xt, double* V, const double* T, const double* Xi, const double* G, const double* wdiag,
                   double* part, int pstride, const SolveState* st, int rfree);

@@ -64,7 +64,6 @@
 
 namespace mbpcg {
 
-constexpr int kMxMinKP = 4;  // narrower blocks have too few FP64 operations per byte
 constexpr int kMxDigits = 7;
 constexpr int kMxThreads = 256;  // threads per CTA
 constexpr int kMxGramBits = 56;  // B of the Grams
@@ -536,7 +535,8 @@ k_gram_mx(int n, const double* __restrict__ X, const double* __restrict__ Y, con
           double* __restrict__ part, int pstride, const SolveState* __restrict__ st) {
   constexpr int KV = 16, WARPS = kMxThreads / 32;
   if (st != nullptr && st->done) return;
-  constexpr bool BAL = !SYM && KP >= KV;  // (a view row is a row of the block)
+  constexpr bool BAL = !SYM;
+  static_assert(SYM || KP >= KV, "a view row is a row of the block");
   __shared__ double red[WARPS][KV * KV];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
   // KP = 32: rows are 32 wide, this problem's columns start at xc (X) and yc (Y)
