@@ -1549,7 +1549,7 @@ size_t mbpcg_k_scratch_bytes(int32_t n, int32_t s) {
   // each) and the CSR one at least as many as the dense one
   Dims dm = make_dims(n, 0, s, MBPCG_ALGO_MBPCG, 0, num_sms()), df = dm;
   apply_mixed(df);
-  return (size_t)(std::max(dm.nbmax, df.nbmax) + 1) * dm.pstride * sizeof(double);
+  return (size_t)std::max(dm.nbmax, df.nbmax) * dm.pstride * sizeof(double);
 }
 
 static int k_product_gram(int dense, int32_t n, const int32_t* rp, const int32_t* ci, const double* av,

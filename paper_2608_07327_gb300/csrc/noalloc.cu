@@ -24,13 +24,12 @@
 namespace {
 
 // Capacity: s <= 16 (partial-slot stride npack(16) + 16 + 1 = 153 -> 156 doubles) and up to 1216
-// CTAs (a sparse product launches up to 8 per SM: 1216 on a 152-SM GB300), plus one slot for the
-// reduced sums: 1217 * 156 doubles = 1 518 816 bytes, held by every GPU that loads the library
-// until exit.
+// CTAs (a sparse product launches up to 8 per SM: 1216 on a 152-SM GB300): 1216 * 156 doubles = 1 517 568
+// bytes, held by every GPU that loads the library until exit.
 constexpr int kMaxS = 16;
 constexpr int kMaxCtas = 1216;
 constexpr int kSlot = 156;
-constexpr size_t kScratchDoubles = (size_t)(kMaxCtas + 1) * kSlot;
+constexpr size_t kScratchDoubles = (size_t)kMaxCtas * kSlot;
 
 static __device__ __align__(256) double g_spmm_gram_scratch[kScratchDoubles];
 
