@@ -664,7 +664,7 @@ int finish_create(mbpcg_ctx* h) {
 // Two columns, long rows, a large system: the Gram by tiles, with fewer registers asked of the rows that live on
 // L1 (27-point, KP = 2, us in registers / by tiles: 60^3 37 / 41, 72^3 77 / 81, 84^3 115 / 102, 96^3 168 / 153;
 // 7-point 128^3 76 / 88).
-bool spmm_by_tiles(const Dims& dm) { return dm.kp == 2 && dm.nnz > 16LL * dm.n && dm.n > 1 << 19; }
+bool spmm_by_tiles(const Dims& dm) { return dm.kp == 2 && long_rows(dm.n, dm.nnz) && dm.n > kGramTilesMinRows; }
 
 void enqueue_product(mbpcg_ctx* h, const RowOps* ops, const double* X, double* Y, int gram, const SolveState* st) {
   const Dims& dm = h->dm;
@@ -682,7 +682,7 @@ void enqueue_product(mbpcg_ctx* h, const RowOps* ops, const double* X, double* Y
     if (gram && dm.mx_gram) ops->product_gram_mx(h->stream, dm.nb_mx, dm.n, X, Y, bal, h->part, dm.pstride, st);
   } else {
     ops->spmm(h->stream, dm.nb, dm.n, h->rp, h->ci, h->av, X, Y, h->part, dm.pstride, st,
-              gram && !dm.mx_gram ? (spmm_by_tiles(dm) ? 2 : 1) : 0);
+              !gram || dm.mx_gram ? kGramNone : spmm_by_tiles(dm) ? kGramTiles : kGramRegisters);
     if (gram && dm.mx_gram) ops->product_gram_mx(h->stream, dm.nb_mx, dm.n, X, Y, bal, h->part, dm.pstride, st);
   }
 }
@@ -855,7 +855,7 @@ void enqueue_cg_setup(mbpcg_ctx* h) {
 // product alone keeps more of them (us, sums apart / in the product): 27-point 40^3 14.6 / 12.8, 48^3 17.5 / 15.8,
 // 56^3 23.1 / 25.5, 72^3 49 / 55, 96^3 102 / 121; 7-point 60^3 12.9 / 12.4, 128^3 65 / 61 (with scaling 70 / 62);
 // apart costs a launch besides.
-bool cg_sums_in_product(const Dims& dm) { return dm.nnz <= 16LL * dm.n || dm.n <= 1 << 17; }
+bool cg_sums_in_product(const Dims& dm) { return !long_rows(dm.n, dm.nnz) || dm.n <= 1 << 17; }
 
 void enqueue_cg_body(mbpcg_ctx* h) {
   const Dims& dm = h->dm;
@@ -1565,7 +1565,7 @@ static int k_product_gram(int dense, int32_t n, const int32_t* rp, const int32_t
     ops->dense(st, dm.nb_dense, n, A, P, AP, nullptr, nullptr);
     ops->gram(st, dm.nb, n, P, AP, part, dm.pstride, nullptr);
   } else {
-    ops->spmm(st, dm.nb, n, rp, ci, av, P, AP, part, dm.pstride, nullptr, 1);
+    ops->spmm(st, dm.nb, n, rp, ci, av, P, AP, part, dm.pstride, nullptr, kGramByRows);
   }
   launch_reduce_gram(st, part, dm.nb, dm.pstride, s, G);
   CUDA_TRY(cudaGetLastError());

@@ -26,11 +26,16 @@ inline cudaError_t ensure_dynamic_smem(K* func, size_t bytes) {
 // block update and the Grams of one block, W/P update, Gram of the product.
 constexpr int kMxMinKP = 4, kMxPwMinKP = 8, kMxProductMinKP = 16;
 
+// How the CSR product forms its Gram matrix: not at all, in registers (the wider blocks: by tiles), by tiles also
+// at KP = 2, or at KP = 2 as the length of the rows asks, which the device looks up (spmm_by_tiles in api.cu).
+enum { kGramNone = 0, kGramRegisters = 1, kGramTiles = 2, kGramByRows = 3 };
+constexpr int kGramTilesMinRows = 1 << 19;
+
 // Host launchers of the row kernels for one padded width KP (defined in inst_kp*.cu).
 struct RowOps {
   int kp;
   void (*spmm)(cudaStream_t, int nb, int n, const int* rp, const int* ci, const double* av, const double* P,
-               double* Q, double* part, int pstride, const SolveState* st, int gram);  // gram 2: by tiles (KP = 2)
+               double* Q, double* part, int pstride, const SolveState* st, int gram);  // gram: kGram...
   // one column: the CG's w = A r with the CTA partials of k_cg_dots
   void (*spmm_dots)(cudaStream_t, int nb, int n, const int* rp, const int* ci, const double* av, const double* r,
                     double* w, const double* wdiag, double* part, int pstride, const SolveState* st);

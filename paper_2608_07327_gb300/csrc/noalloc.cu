@@ -120,7 +120,7 @@ extern "C" int mbpcg_k_spmm_gram_noalloc(int32_t n, const int32_t* row_ptr, cons
   // Every partial slot the reduction reads (nb of them) is fully written by this call's product
   // kernel first, so nothing in the array has to start at zero.
   cudaStream_t st = (cudaStream_t)stream;
-  mbpcg::row_ops(kp)->spmm(st, nb, n, row_ptr, col_idx, vals, P, AP, scratch, kSlot, nullptr, 1);
+  mbpcg::row_ops(kp)->spmm(st, nb, n, row_ptr, col_idx, vals, P, AP, scratch, kSlot, nullptr, mbpcg::kGramByRows);
   mbpcg::launch_reduce_gram(st, scratch, nb, kSlot, s, G);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess)

@@ -16,7 +16,9 @@ namespace mbpcg {
 // when GRAM, the CTA partials of the upper triangle of P^T Q (the Gram that defines Xi), so that
 // A P is never read back. Threads own CPT consecutive columns of a row; the row of P that a
 // nonzero selects is KP*8 contiguous bytes, read with 16-byte vector loads.
-template <int KP, bool GRAM, bool TILES = false>
+// ROUTE: of the two forms of a Gram (TILES), only the one for this matrix does anything; its entries are counted
+// here, where the caller has them on the device only (the form that returns takes 2 us).
+template <int KP, bool GRAM, bool TILES = false, bool ROUTE = false>
 __global__ void __launch_bounds__(kThreads)
 k_spmm(int n, const int* __restrict__ rp, const int* __restrict__ ci, const double* __restrict__ av,
        const double* __restrict__ P, double* __restrict__ Q, double* __restrict__ part, int pstride,
@@ -24,6 +26,9 @@ k_spmm(int n, const int* __restrict__ rp, const int* __restrict__ ci, const doub
   using C = Cfg<KP>;
   using G = GramTile<KP>;
   if (st != nullptr && st->done) return;
+  if constexpr (ROUTE) {
+    if (long_rows(n, __ldg(rp + n)) != TILES) return;
+  }
   // A thread that has whole rows (KP <= 4) sums the Gram's terms of its rows in registers: KP (KP + 1) / 2 FMAs
   // a row and no barrier (diffusion 128^3, KP = 4: 148 us with the Gram against 167 by tiles; 129 us of
   // the FP64 pipe; KP = 2 89 -> 77, KP = 1 59 -> 50; Poisson 160^2, KP = 4 11.5 -> 9.0);
