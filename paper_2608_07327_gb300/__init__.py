@@ -165,17 +165,18 @@ class Solver:
         """Solve A x = b. b (and U, n x s column-major) are numpy arrays (host path, mbpcg_solve)
         or torch CUDA tensors (device path, mbpcg_solve_dev). Returns (x, info dict)."""
         import torch
-        self.stream.wait_stream(torch.cuda.current_stream())
         if hasattr(b, "is_cuda") and b.is_cuda:
             x = torch.empty(self.n, dtype=torch.float64, device=b.device)
             Ud = None
             if U is not None:
                 Ud = U.t().contiguous() if U.dim() == 2 else U  # column-major n x s == row-major s x n
+            self.stream.wait_stream(torch.cuda.current_stream())  # after the copy of U that the line above enqueues
             st, info = mbpcg_solve_dev(self.h, b, Ud, tol, maxit, x)
         else:
             b = np.ascontiguousarray(b, dtype=np.float64)
             Uh = None if U is None else np.asfortranarray(U, dtype=np.float64)
             x = np.zeros(self.n)
+            self.stream.wait_stream(torch.cuda.current_stream())
             st, info = mbpcg_solve(self.h, b, Uh, tol, maxit, x)
         if st not in (MBPCG_OK, MBPCG_NOT_CONVERGED, MBPCG_BREAKDOWN):
             raise MBPCGError(st, "mbpcg_solve")
