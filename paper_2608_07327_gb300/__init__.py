@@ -142,6 +142,8 @@ class Solver:
         else:
             nbytes = mbpcg_workspace_size_csr(self.n, int(A.row_ptr[-1]), self.s, algo, precision)
         self.workspace = torch.empty(nbytes, dtype=torch.uint8, device="cuda")
+        # the allocator may hand out memory that work of the caller's stream still uses
+        self.stream.wait_stream(torch.cuda.current_stream())
         if self.dense:
             a = np.asfortranarray(A.a, dtype=np.float64)
             self.h = mbpcg_create_dense(self.n, a, self.s, precond, algo, precision, seed, 0, self.workspace, nbytes,

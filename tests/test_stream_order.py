@@ -1,12 +1,16 @@
-"""Solver.solve on device tensors: the copy that turns U into columns is enqueued on the caller's stream, so the
-handle's stream has to wait for that stream after the copy and before the solve. Read from the order of the calls, on
-the CPU, with the streams and the library call replaced by recorders."""
+"""The handle's stream waits for the caller's after what the caller's stream still has to do for the call: the copy that
+turns U into columns (Solver.solve on device tensors), and whatever used the workspace's memory before (Solver). Read
+from the order of the calls, on the CPU, with the streams and the library calls replaced by recorders."""
 import pytest
+
+import workloads as wl
 
 torch = pytest.importorskip("torch")
 
 
 class Recorder:
+    cuda_stream = 0
+
     def __init__(self, log):
         self.log = log
 
@@ -49,3 +53,18 @@ def test_the_handle_waits_for_the_copy_of_u(monkeypatch, dims):
     monkeypatch.setattr(mb, "mbpcg_solve_dev", solve_dev)
     sv.solve(DeviceVector(), None if dims is None else Block(log, dims))
     assert log == (["copy of U"] if dims == 2 else []) + ["wait", "solve"]
+
+
+@pytest.mark.parametrize("dense", [False, True])
+def test_the_handle_waits_for_the_memory_of_its_workspace(monkeypatch, dense):
+    import paper_2608_07327_gb300 as mb
+    log = []
+    monkeypatch.setattr(torch.cuda, "is_available", lambda: True)
+    monkeypatch.setattr(torch.cuda, "Stream", lambda: Recorder(log))
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda *a: None)
+    monkeypatch.setattr(torch, "empty", lambda *a, **k: log.append("workspace"))
+    for kind in ("csr", "dense"):
+        monkeypatch.setattr(mb, "mbpcg_workspace_size_" + kind, lambda *a: 256)
+        monkeypatch.setattr(mb, "mbpcg_create_" + kind, lambda *a: log.append("create"))
+    mb.Solver(wl.dense_mtm(4, 1) if dense else wl.poisson2d(3))
+    assert log == ["workspace", "wait", "create"]
