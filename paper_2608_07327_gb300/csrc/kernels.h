@@ -31,6 +31,9 @@ constexpr int kMxMinKP = 4, kMxPwMinKP = 8, kMxProductMinKP = 16;
 enum { kGramNone = 0, kGramRegisters = 1, kGramTiles = 2, kGramByRows = 3 };
 constexpr int kGramTilesMinRows = 1 << 19;
 
+// Long rows: more than 16 entries on average. Their entries live on L1.
+__host__ __device__ inline bool long_rows(int n, long long nnz) { return nnz > 16LL * n; }
+
 // Host launchers of the row kernels for one padded width KP (defined in inst_kp*.cu).
 struct RowOps {
   int kp;

@@ -78,9 +78,6 @@ __device__ inline void punpack(int e, int& l, int& j) {
   l = e - j * (j + 1) / 2;
 }
 
-// Long rows: more than 16 entries on average. Their entries live on L1.
-__host__ __device__ inline bool long_rows(int n, long long nnz) { return nnz > 16LL * n; }
-
 // Balanced contiguous row range of this CTA.
 __device__ inline void row_range(int n, int& r0, int& r1) {
   r0 = (int)(((long long)n * blockIdx.x) / gridDim.x);

@@ -6,6 +6,7 @@
 // once when the solve has finished (SolveState::done), so a CUDA-graph loop body costs nothing
 // after convergence.
 #pragma once
+#include "kernels.h"
 #include "mbpcg_device.cuh"
 #include "tma.cuh"
 
@@ -142,8 +143,9 @@ k_spmm_dots(int n, const int* __restrict__ rp, const int* __restrict__ ci, const
 // (half of them at n = 2304, KP = 8: 100 us; now 76 us, of which 69 are the FP64 pipe's;
 // n = 4096, KP = 4: 139 -> 119; KP = 32: 916 -> 898; n = 900, KP = 32: 132 -> 60).
 // Rows of odd length (n odd) break the 16-byte rule of bulk copies; then the same
-// pipeline is filled by 8-byte asynchronous copies (cp.async; n = 4097, KP = 8: 336 -> 233 us). Every mbarrier wait is bounded: on a timeout the CTA sets
-// *err (if given), waits (bounded) for the copies it still has in flight, and returns.
+// pipeline is filled by 8-byte asynchronous copies (cp.async; n = 4097, KP = 8: 336 -> 233 us). Every mbarrier wait
+// is bounded: on a timeout the CTA sets *err (if given), waits (bounded) for the copies it still has in flight, and
+// returns.
 template <int KP, int TR>
 struct DenseCfg {
   static constexpr int G = 4 * TR;
@@ -467,8 +469,9 @@ k_axpy(int n, const double* __restrict__ P, const double* __restrict__ Q, const 
   }
   int r0, r1;
   row_range(n, r0, r1);
-  // whole rows: Gram terms and norms in registers, as in k_spmm (Poisson 160^2, KP = 4: 15.8 -> 14.1 us; 36^3,
-  // KP = 2, implicit residual 13.8 -> 8.1; diffusion 128^3, KP = 2 96 -> 86, KP = 1 29.6 -> 30.5)
+  // whole rows: Gram terms and norms in registers, as in k_spmm (us by tiles / in registers: Poisson 160^2, KP = 4 15.8
+  // / 14.1; 36^3, KP = 2, implicit residual 13.8 / 8.1; diffusion 128^3, KP = 2 96 / 86; KP = 1: 48^3 8.6 / 7.0, 96^3
+  // 16.6 / 15.9, 128^3 33.0 / 31.0 with scaling and 29.5 / 30.5 without, implicit 64^3 11.5 / 8.7)
   if constexpr (kRegs) {
     __syncthreads();
     double sum[NS];
