@@ -58,10 +58,15 @@ typedef enum { MBPCG_PRECOND_NONE = 0, MBPCG_PRECOND_JACOBI = 1 } mbpcg_precond;
  * paper's baseline, Section 4), s ignored. */
 typedef enum { MBPCG_ALGO_MBPCG = 0, MBPCG_ALGO_CG = 1 } mbpcg_algo;
 
-/* Arithmetic of the n-proportional work. FP64: everything in double precision, on the FP64 pipe; in CSR
- * MBPCG solves with at least 2^17 values per padded block (n times the padded width, width >= 4) the block
- * update, and for wider blocks the W/P update and the Gram matrices, form their s x s contractions by
- * exact digit splitting on the tensor cores, with the accuracy of an FP64 sum (csrc/rows_mma.cuh).
+/* Arithmetic of the n-proportional work. FP64: everything in double precision, on the FP64 pipe, but for the
+ * s x s contractions of large CSR MBPCG solves, which are formed by digit splitting on the tensor cores
+ * (csrc/rows_mma.cuh): from padded width 4 and 2^17 values per block (n times the padded width) those of the
+ * block update, of V^T V and of the set-up and exit Grams; from width 8 those of the W/P update; from width 16 and
+ * 2^19 values P^T (A P). An entry of a row product sum_l x_il m_lj is then off by about 2^-57 sqrt(s) of
+ * max_l |x_il| / c_l times max_l c_l |m_lj| and its rounding, where c_l is the size of column l as P^T A P, zeta or
+ * Sigma has it (1 for P): no more than the s roundings of an FP64 sum wherever the columns of a row are of like
+ * size but for c, and not term by term, as those are. A Gram entry is off by about 2^-56 of the largest
+ * products of its rows, added like n random numbers, P^T (A P) with its rows balanced by the diagonal of A.
  * MIXED_FP32 (MBPCG only; CSR or dense A): the inner solves keep the n x s blocks and the (scaled)
  * matrix in FP32 (a dense A adds an FP32 copy, n x round_up(n, 32) floats, to the workspace) and do
  * the products and block updates in FP32 with FP32 accumulation; the s x s

@@ -82,8 +82,8 @@ __device__ __forceinline__ void dot2_add(float& s, float& c, float x, float y) {
 }
 
 // Two FP32 numbers in one register pair, for the packed FP32 instructions: the same roundings as the scalar
-// ones with half the instructions to issue (27-point 96^3, KP = 16: the block update 169 -> 154 us, the Gram of
-// the product 64.6 -> 63.7).
+// ones with half the instructions to issue (27-point 96^3, KP = 16: the block update 169 -> 152 us, the Gram of
+// the product 64.6 -> 62).
 struct f32x2 {
   unsigned long long v;
 };

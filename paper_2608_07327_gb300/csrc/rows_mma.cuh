@@ -1,34 +1,33 @@
 // The row passes of the CSR handles (block update, W/P update, Gram matrices) on the FP16 tensor cores
-// with FP64 accuracy, by exact digit splitting (Ozaki et al., "Error-free transformations of matrix
-// multiplication by using fast routines of matrix multiplication and its applications", Numer.
-// Algorithms 2012), from registers to registers (mma.sync.m16n8k16).
+// with the precision of FP64 blocks (the bounds stand below), by digit splitting (Ozaki et al., "Error-free
+// transformations of matrix multiplication by using fast routines of matrix multiplication and its
+// applications", Numer. Algorithms 2012), from registers to registers (mma.sync.m16n8k16).
 //
 // Why. GB300 issues 2 FP64 lanes per clock per SM: at 16 columns a row of the block update is 768 + 144
 // FP64 FMAs, and the FP64 pipe made these passes 10 times slower than their bytes. Here the contractions
 // are integer digit products on the tensor cores, the splitting and recombination are integer
 // operations, and the FP64 pipe keeps one add per output and the norms; the three pipes run side by
-// side. What binds now is the integer work: about 50 operations per value split or combined, half of them
-// on the 16-lane ALU (54 % busy). Measured (us per launch, FP64 pipe -> here; the block update with its
-// Gram V^T V):
+// side. What binds now is the integer work: about 50 operations per value split or combined. Measured (us per
+// launch, FP64 pipe -> here; the block update with its Gram V^T V):
 //                                    block update        W/P update     Gram P^T (A P) (in the product)
-//   27-point 96^3, KP = 16          1357 -> 258 + 66     408 -> 153      239 -> 131
-//   diffusion 64^3, KP = 32         1619 -> 283 + 116    471 -> 160      280 -> 126
-//   diffusion 100^3, KP = 8          455 -> 145 + 55     129 -> 88        78 -> 97 (kept fused)
-//   diffusion 128^3, KP = 4          288 -> 157 + 52      77 -> 92 (kept)  58 -> 110 (kept fused)
+//   27-point 96^3, KP = 16          1357 -> 234 + 65     408 -> 147      239 -> 124 (102 without balancing)
+//   diffusion 64^3, KP = 32         1619 -> 299 + 111    471 -> 165      280 -> 128
+//   diffusion 100^3, KP = 8          455 -> 140 + 49     129 -> 85        78 -> 97 (kept fused)
+//   diffusion 128^3, KP = 4          288 -> 152 + 50      77 -> 92 (kept)  58 -> 110 (kept fused)
 // The same contractions in fixed point on the integer pipe (two 28-bit limbs, three IMAD.WIDE a term; 62
-// lanes per clock per SM) took 383 + 115 and 205 us at KP = 16. The tile shapes (16 rows, 16 columns at most) are those of mma.sync: a warp holds its operands
-// and results in registers in the layout in which it reads and writes them, so that there is no
-// staging, no shared memory but the k x k matrices' digits, and no barrier in the loops (tcgen05.mma's
-// smallest tile of 128 rows, with its operands in shared memory and results in tensor memory, needs
-// all of these).
+// lanes per clock per SM) took 383 + 115 and 205 us at KP = 16. The tile shapes (16 rows, 16 columns at most) are
+// those of mma.sync: a warp holds its operands and results in registers in the layout in which it reads and
+// writes them, so that there is no staging, no shared memory but the k x k matrices' digits, and no barrier in the
+// loops (tcgen05.mma's smallest tile of 128 rows, with its operands in shared memory and results in tensor memory,
+// needs all of these).
 //
 // Digits. A group of values (a row of a block, a column of a k x k matrix, a column of the rows that a
 // warp sums) whose largest biased exponent is E is written x = 2^(E - 1022) 2^-B X, X the nearest
 // integer (|X| <= 2^B: the group's largest value keeps all its bits, any other loses what lies below
 // 2^-(B+1) of the scale), and X in 7 base-256 digits: six of -128..127 (X plus 128 in every digit, minus
 // 128 digit by digit) and a leading one of at most 2^(B-48), all exact in FP16. Digit pairs (t, u) are kept
-// for t + u <= 6 (28 products); what is dropped is random, about 2^-58 of the two scales for each root of
-// a term at B = 57. (At B = 56 it is four times, at B = 55 sixteen times that: V zeta^-1 at KP = 32 was off by
+// for t + u <= 6 (28 products); what is dropped is random, 2^-60 of the two scales times the root of the number
+// of terms at B = 57. (At B = 56 it is four times, at B = 55 sixteen times that: V zeta^-1 at KP = 32 was off by
 // 8e-17 and 2.6e-16 of its norm, the FP64 pass by 5.2e-17 and B = 57 by 5.1e-17; at B = 57 no product of any
 // width was further off than the FP64 pass on the Poisson, diffusion and 27-point systems, in an emulation.)
 // (With one side's digits 0..255, two operations fewer per pair of digits, what is dropped has a mean
@@ -36,15 +35,16 @@
 // state after 8 iterations of the 27-point stencil was 100 times further off.)
 //   A level sum S_L = sum_{t+u=L} sum_l is exact in the FP32 accumulator: within 2^18 * 16 = 2^22 (level 0) and
 // (2 * 2^16 + 5 * 2^14) * 16 < 2^22 over one mma step of a row product at B = 57 (KP = 32 takes the levels of its
-// two steps out one after the other); below (2 * 2^15 + 5 * 2^14) * 112 rows < 2^24 in a Gram (B = 56) between two drains.
+// two steps out one after the other); below (2 * 2^15 + 5 * 2^14) * 112 rows < 2^24 in a Gram
+// (B = 56) between two drains.
 //   A row product is off by 2^-58 or so of max_l |x_il| max_l |m_lj|, an FP64 sum by 2^-53 of sum_l |x_il m_lj|.
 // These differ where columns of the block differ in size and the matrix makes up for it. V is such a block (a
 // column whose Cholesky factor is 10^-6 of the others'), so is R at the set-up with a graded U, and A P, where a
-// smooth column of P has eigenvalues far below the others': there column l enters as 2^o V_l, and row l of the
-// matrix as 2^-o of it, with o from the norms of the columns. The k x k steps know them: zeta has the column norms of V,
-// Sigma those of R, and P^T A P = W^T (A P) is A P projected on the orthonormal W (emulated, Poisson 183^2, one smooth
-// column and three rough ones: (A P) T off by 7e-14 of its norm without and 5e-17 with them, FP64 sums 9e-17).
-// P has none: its columns are W's, of norm 1, and what CG adds to them.
+// smooth column of P has eigenvalues far below the others': there column l enters as 2^o of it, and row l of the
+// matrix as 2^-o, with o from the norms of the columns. The k x k steps know them: zeta has the column norms of
+// V, Sigma those of R, and P^T A P = W^T (A P) is A P projected on the orthonormal W (emulated, Poisson 183^2, one
+// smooth column and three rough ones: (A P) T off by 7e-14 of its norm without and 5e-17 with them, FP64 sums
+// 9e-17). P has none: its columns are W's, of norm 1, and what CG adds to them.
 //
 // Widths. The row products see the block as rows of KV = max(KP, 8) columns and a Gram as rows of 16: for
 // a narrower block several rows make one, with the k x k matrix repeated on the diagonal (the diagonal
@@ -362,8 +362,8 @@ __device__ __forceinline__ void mx_store_rows(double* X, size_t row, size_t nf, 
 }
 
 // Block update of Algorithm 1 (as k_axpy): X~ += P T, R -= (A P) T, V = W - (A P) Xi, and the CTA partials
-// of nu at part[NPACK + j]. Gp: the upper triangle of P^T (A P). RFREE: R is neither read nor written, and there are no norms. Tiles of 16
-// view rows are dealt to the warps of the grid in turn (their sums do not depend on the order).
+// of nu at part[NPACK + j]. Gp: the upper triangle of P^T (A P). RFREE: R is neither read nor written, and there are
+// no norms. Tiles of 16 view rows are dealt to the warps of the grid in turn (their sums do not depend on the order).
 template <int KP, bool RFREE>
 __global__ void __launch_bounds__(kMxThreads, KP >= 32 ? 1 : 2)
 k_axpy_mx(int n, const double* __restrict__ P, const double* __restrict__ Q, const double* __restrict__ W,
@@ -515,18 +515,20 @@ k_pw_mx(int n, const double* __restrict__ V, double* __restrict__ W, double* __r
 
 // ------------------------------------------------------------------------------------ Gram matrices
 
-// CTA partials of the upper triangle of X^T Y (Y = X when SYM). WT: of X^T D^2 X,
-// with D in dw and as (D X)^T (D X) up to KP = 16, where that leaves one block to split (diffusion 77^3: 56 us
-// against 80 for (D^2 X)^T X), and D^2 in dw at KP = 32, where there are two anyway (FP64 products). A warp keeps its own column scales: the mma takes 16 view rows as its reduction index, so that a
-// lane holds the view columns g and g + 8 of 4 rows, as the left operand and as the right one alike. The
-// scales only grow; a tile that exceeds them (the first one, and then rarely: one bit of headroom) first
-// has the sums turned into FP64. 56 bits of the scale: with 55 the Grams of unscaled diffusion
-// were off by up to 1.5 times what FP64 sums are, with 56 by less than those on every system (in an emulation).
-// X^T Y of two blocks is P^T (A P). Where the diagonal of A varies, P is small where A P is large, and a scale over
-// the rows would lose what their product does not: the rows are balanced by r = half the exponent of a_ii (dw,
-// or NULL; to that of a_00, at most 63), 2^r X against 2^-r Y. (Two unknowns per point in units 10^6 apart, 16
-// columns, emulated: off by 2e-12 of the largest entry without and 1e-16 with it, FP64 sums by 1e-15.) KP = 32 is three problems of 16 columns (blockIdx.y: columns 0..15 with
-// themselves, with 16..31, and 16..31 with themselves).
+// CTA partials of the upper triangle of X^T Y (Y = X when SYM). WT: of X^T D^2 X, with D in dw and as
+// (D X)^T (D X) up to KP = 16, where that leaves one block to split (diffusion 77^3: 56 us against 80 for
+// (D^2 X)^T X; D x is rounded once more than D^2 x, 2^-53 of each term), and D^2 in dw at KP = 32, where there are
+// two anyway (FP64 products). A warp keeps its own column scales: the mma takes 16 view rows as its reduction
+// index, so that a lane holds the view columns g and g + 8 of 4 rows, as the left operand and as the right one
+// alike. The scales only grow; a tile that exceeds them (the first one, and then rarely: one bit of headroom)
+// first has the sums turned into FP64. 56 bits of the scale: with 55 the Grams of unscaled diffusion were off by up
+// to 1.5 times what FP64 sums are, with 56 by less than those on every system (in an emulation). KP = 32 is three
+// problems of 16 columns (blockIdx.y: columns 0..15 with themselves, with 16..31, and 16..31 with themselves).
+//   X^T Y of two blocks is P^T (A P). Where the diagonal of A varies, P is small where A P is large, and a scale over
+// the rows would lose what their product does not: the rows are balanced by r = half the exponent of a_ii (dw, or
+// NULL; relative to a_00, at most 63), 2^r X against 2^-r Y. (Two unknowns per point in units 10^6 apart, 16 columns,
+// emulated: off by 2e-12 of the largest entry without and 1e-16 with it, FP64 sums by 1e-15. The kernel takes 124
+// us with it on the 27-point system, 102 without.)
 constexpr int kMxDrainTiles = 7;  // 112 rows between two drains of the FP32 sums into FP64
 
 template <int KP, bool SYM, bool WT = false>
