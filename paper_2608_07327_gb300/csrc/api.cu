@@ -248,6 +248,7 @@ struct mbpcg_ctx {
   // device pointers
   int *rp, *ci, *flag;
   double *av, *A, *diag, *d, *sqd, *wdiag, *b, *rhs, *bs, *x, *xbest;
+  int* rexp;  // row exponents of the product's Gram on the tensor cores (k_row_exponents), or NULL
   double *U, *X0, *Xt, *R, *W, *P, *Q, *V;
   double *r, *w, *xb, *p, *sv;
   double *r2, *w2, *sv2;
@@ -614,6 +615,11 @@ int finish_create(mbpcg_ctx* h) {
     CUDA_TRY(cudaGetLastError());
     h->wdiag = h->diag;
   } else {
+    if (h->dm.mx_gram) {  // (a scaled A has ones on its diagonal) in the place of sqd, which is not used without scaling
+      h->rexp = reinterpret_cast<int*>(h->sqd);
+      k_row_exponents<<<g, 256, 0, h->stream>>>(n, h->diag, h->rexp);
+      CUDA_TRY(cudaGetLastError());
+    }
     h->d = nullptr;
     h->sqd = nullptr;
     h->wdiag = nullptr;
@@ -668,7 +674,6 @@ bool spmm_by_tiles(const Dims& dm) { return dm.kp == 2 && long_rows(dm.n, dm.nnz
 
 void enqueue_product(mbpcg_ctx* h, const RowOps* ops, const double* X, double* Y, int gram, const SolveState* st) {
   const Dims& dm = h->dm;
-  const double* bal = h->wdiag == nullptr ? h->diag : nullptr;  // balances the Gram's rows; a scaled A has ones there
   if (dm.dense && dm.tc) {
     // the loop's product reads P, whose column exponents the W/P update has already formed
     oz_product(h->stream, dm.n, dm.kp, dm.sms, h->oz_a, h->oz_ea, X, h->oz_p, h->oz_ep, h->oz_q, Y, &h->st->kerr, st,
@@ -679,11 +684,11 @@ void enqueue_product(mbpcg_ctx* h, const RowOps* ops, const double* X, double* Y
   } else if (h->prod64 == MBPCG_PRODUCT_CSR_TILED) {
     spmm_tiled(h->stream, dm.kp, dm.nb, dm.n, h->rp, h->av, h->plan, X, Y, h->part, dm.pstride, st,
                gram && !dm.mx_gram);
-    if (gram && dm.mx_gram) ops->product_gram_mx(h->stream, dm.nb_mx, dm.n, X, Y, bal, h->part, dm.pstride, st);
+    if (gram && dm.mx_gram) ops->product_gram_mx(h->stream, dm.nb_mx, dm.n, X, Y, h->rexp, h->part, dm.pstride, st);
   } else {
     ops->spmm(h->stream, dm.nb, dm.n, h->rp, h->ci, h->av, X, Y, h->part, dm.pstride, st,
               !gram || dm.mx_gram ? kGramNone : spmm_by_tiles(dm) ? kGramTiles : kGramRegisters);
-    if (gram && dm.mx_gram) ops->product_gram_mx(h->stream, dm.nb_mx, dm.n, X, Y, bal, h->part, dm.pstride, st);
+    if (gram && dm.mx_gram) ops->product_gram_mx(h->stream, dm.nb_mx, dm.n, X, Y, h->rexp, h->part, dm.pstride, st);
   }
 }
 

@@ -72,11 +72,11 @@ struct RowOps {
   void (*pw_pre)(cudaStream_t, int n, const double* VZi, const double* PZt, double* W, double* P, const SolveState* st,
                  int* emax);
   // the row passes on the tensor cores (NULL below their widths): the Gram X^T D^2 X (D and D^2, or NULL), the
-  // product's Gram P^T Q (diag: balances the rows, or NULL), the block update without its Gram (G: P^T A P,
+  // product's Gram P^T Q (rexp: balances the rows, or NULL), the block update without its Gram (G: P^T A P,
   // packed), the W/P update (setp: Z is the Cholesky factor Sigma of V)
   void (*gram_mx)(cudaStream_t, int nb, int n, const double* X, const double* d, const double* d2, double* part,
                   int pstride, const SolveState* st);
-  void (*product_gram_mx)(cudaStream_t, int nb, int n, const double* P, const double* Q, const double* diag,
+  void (*product_gram_mx)(cudaStream_t, int nb, int n, const double* P, const double* Q, const int* rexp,
                           double* part, int pstride, const SolveState* st);
   void (*axpy_mx)(cudaStream_t, int nb, int n, const double* P, const double* Q, const double* W, double* R,
                   double* Xt, double* V, const double* T, const double* Xi, const double* G, const double* wdiag,
@@ -171,6 +171,7 @@ __global__ void k_small_cg(SolveState* st, const double* part, int nparts, int p
                            int use_cond);
 __global__ void k_validate_csr(int n, long long nnz, const int* rp, const int* ci, int* flag);
 __global__ void k_diag_csr(int n, const int* rp, const int* ci, const double* av, double* diag, int* flag);
+__global__ void k_row_exponents(int n, const double* diag, int* rexp);
 __global__ void k_diag_dense(int n, const double* A, double* diag, int* flag);
 __global__ void k_check_finite(long long count, const double* v, int* flag);
 __global__ void k_make_scaling(int n, const double* diag, double* d, double* sqd);

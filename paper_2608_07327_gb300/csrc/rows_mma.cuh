@@ -10,8 +10,8 @@
 // side. What binds now is the integer work: about 50 operations per value split or combined. Measured (us per
 // launch, FP64 pipe -> here; the block update with its Gram V^T V):
 //                                    block update        W/P update     Gram P^T (A P) (in the product)
-//   27-point 96^3, KP = 16          1357 -> 234 + 65     408 -> 147      239 -> 124 (102 without balancing)
-//   diffusion 64^3, KP = 32         1619 -> 299 + 111    471 -> 165      280 -> 128
+//   27-point 96^3, KP = 16          1357 -> 234 + 65     408 -> 147      239 -> 108 (102 without balancing)
+//   diffusion 64^3, KP = 32         1619 -> 299 + 111    471 -> 165      280 -> 125
 //   diffusion 100^3, KP = 8          455 -> 140 + 49     129 -> 85        78 -> 97 (kept fused)
 //   diffusion 128^3, KP = 4          288 -> 152 + 50      77 -> 92 (kept)  58 -> 110 (kept fused)
 // The same contractions in fixed point on the integer pipe (two 28-bit limbs, three IMAD.WIDE a term; 62
@@ -52,7 +52,7 @@
 // different units, and a row 10^6 below its neighbour would lose 20 bits to a common one.
 //
 // A group that holds an infinity or a NaN has E = kMxNaN, and what is formed from it is NaN. A group below
-// 2^-831 counts as zero (the solver squares norms: it can use nothing below 2^-511).
+// 2^-958 counts as zero (the solver squares norms: it can use nothing below 2^-511).
 #pragma once
 #include <cuda_fp16.h>
 #include <stdint.h>
@@ -68,21 +68,22 @@ constexpr int kMxDigits = 7;
 constexpr int kMxThreads = 256;  // threads per CTA
 constexpr int kMxGramBits = 56;  // B of the Grams
 constexpr unsigned kMxAll = 0xffffffffu;
-constexpr int kMxTiny = 192;    // a group with a scale exponent below this one counts as zero
+constexpr int kMxTiny = 64;     // a group with a scale exponent below this one counts as zero
 constexpr int kMxNaN = 0x4000;  // scale exponent of a group that is not finite
 
 __device__ __forceinline__ int mx_exponent(double x) { return (__double2hiint(x) >> 20) & 0x7FF; }
 
-// X of 2^o x (-128 < o < 128) in a group of scale exponent E (>= its own), to nearest (halves away from zero).
+// X of 2^o x in a group of scale exponent E (>= its own), to nearest (halves away from zero). A group with E below
+// `tiny` is zero; tiny - o >= 64.
 template <int B>
-__device__ __forceinline__ long long mx_int(double x, int E, int o = 0) {
+__device__ __forceinline__ long long mx_int(double x, int E, int o, int tiny) {
   const int h = __double2hiint(x), e = (h >> 20) & 0x7FF;
   // 53 bits moved up to B + 1 (one below the unit), then down to the group's scale;
-  // shr.u64 gives 0 from 64 on, which a zero or subnormal x (e = 0) reaches since E >= 192
+  // shr.u64 gives 0 from 64 on, which a zero or subnormal x (e = 0) reaches since E - o >= 64
   const unsigned long long m = (((unsigned long long)(unsigned)((h & 0xFFFFF) | 0x100000) << 32) |
                                 (unsigned)__double2loint(x)) << (B - 52);
   unsigned long long r;
-  asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(m), "r"((E < kMxTiny ? 4096 : E) - e - o));
+  asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(m), "r"((E < tiny ? 4096 : E) - e - o));
   r = (r + 1) >> 1;
   const long long s = h >> 31;
   return (long long)(r ^ (unsigned long long)s) - s;
@@ -189,9 +190,9 @@ constexpr unsigned long long kMxStartSum =
     (unsigned long long)(kMxStart >> 8) + (unsigned long long)kMxStart * (1ull + 256ull + 65536ull + 16777216ull) +
     ((unsigned long long)(uint32_t)(kMxStart + (kMxStart << 8)) << 32);
 
-// Exponents o[l] (0 to 63) that bring columns l of a block to like size, from a k x k matrix src(j, l) whose
-// columns have the norms of the block's: the largest column has 0 (all threads; the caller synchronises before
-// and after).
+// Exponents o[l] (-63 to 0) that bring columns l of a block to like size, from a k x k matrix src(j, l) whose
+// columns have the norms of the block's: the smallest column that is not zero has 0 (all threads; the caller
+// synchronises before and after).
 template <int KP, typename F>
 __device__ void mx_column_exponents(F src, int (&o)[KP]) {
   __shared__ int c[KP];
@@ -204,10 +205,10 @@ __device__ void mx_column_exponents(F src, int (&o)[KP]) {
   }
   __syncthreads();
   if (tid < KP) {
-    int m = 0;
+    int m = 0x7FF;
 #pragma unroll 8
-    for (int j = 0; j < KP; ++j) m = max(m, c[j]);
-    o[tid] = min(m - c[tid], 63);
+    for (int j = 0; j < KP; ++j) m = c[j] > 0 ? min(m, c[j]) : m;
+    o[tid] = c[tid] > 0 ? max(m - c[tid], -63) : 0;
   }
 }
 
@@ -224,7 +225,7 @@ __device__ void mx_load_matrix(F src, const int* o, MxMatrix<KP>& M) {
     for (int l = 0; l < KP; ++l) {
       const int x = mx_exponent(src(l, tid));
       bad |= x == 0x7FF;
-      e = max(e, x - (o != nullptr ? o[l] : 0));
+      e = max(e, x > 0 && o != nullptr ? x - o[l] : x);
     }
     M.e[tid] = bad ? kMxNaN : e;
   }
@@ -234,9 +235,9 @@ __device__ void mx_load_matrix(F src, const int* o, MxMatrix<KP>& M) {
     const int n = 8 * nb + (lane >> 2), k0 = 16 * ks + 2 * (lane & 3);
     // view matrix: KP x KP blocks on the diagonal
     auto at = [&](int k) {
-      return (k < W::KV && k / KP == n / KP)
-                 ? mx_int<W::B>(src(k % KP, n % KP), M.e[n % KP], o != nullptr ? -o[k % KP] : 0)
-                 : 0LL;
+      if (k >= W::KV || k / KP != n / KP) return 0LL;
+      const double x = src(k % KP, n % KP);
+      return mx_int<W::B>(x, M.e[n % KP], mx_exponent(x) > 0 && o != nullptr ? -o[k % KP] : 0, kMxTiny);
     };
     uint32_t d0[kMxDigits], d1[kMxDigits];
     mx_digits(at(k0), at(k0 + 1), d0);
@@ -283,7 +284,7 @@ struct MxTile {
 #pragma unroll
       for (int r = 0; r < 2; ++r)
         if (e[r] == 0x7FF) e[r] = kMxNaN;
-    } else if (__any_sync(kMxAll, max(e[0], e[1]) >= 0x7FF)) {  // not finite, or large values of a column that o raises
+    } else if (__any_sync(kMxAll, max(e[0], e[1]) >= 0x7FF - 63)) {  // not finite, which o may hide, or large
 #pragma unroll
       for (int r = 0; r < 2; ++r)
         if (largest(r, true) == 0x7FF) e[r] = kMxNaN;
@@ -293,7 +294,7 @@ struct MxTile {
 #pragma unroll
       for (int c = 0; c < W::NB; ++c) {
         uint32_t d[kMxDigits];
-        mx_digits(mx_int<W::B>(v[c][r].x, e[r], ox[c]), mx_int<W::B>(v[c][r].y, e[r], oy[c]), d);
+        mx_digits(mx_int<W::B>(v[c][r].x, e[r], ox[c], kMxTiny), mx_int<W::B>(v[c][r].y, e[r], oy[c], kMxTiny), d);
 #pragma unroll
         for (int t = 0; t < kMxDigits; ++t) a[t][2 * c + r] = d[t];
       }
@@ -525,16 +526,16 @@ k_pw_mx(int n, const double* __restrict__ V, double* __restrict__ W, double* __r
 // to 1.5 times what FP64 sums are, with 56 by less than those on every system (in an emulation). KP = 32 is three
 // problems of 16 columns (blockIdx.y: columns 0..15 with themselves, with 16..31, and 16..31 with themselves).
 //   X^T Y of two blocks is P^T (A P). Where the diagonal of A varies, P is small where A P is large, and a scale over
-// the rows would lose what their product does not: the rows are balanced by r = half the exponent of a_ii (dw, or
-// NULL; relative to a_00, at most 63), 2^r X against 2^-r Y. (Two unknowns per point in units 10^6 apart, 16 columns,
-// emulated: off by 2e-12 of the largest entry without and 1e-16 with it, FP64 sums by 1e-15. The kernel takes 124
-// us with it on the 27-point system, 102 without.)
+// the rows would lose what their product does not: the rows are balanced by r = half the exponent of a_ii
+// (rexp, k_row_exponents; or NULL), 2^r X against 2^-r Y. (Two unknowns per point in units 10^6 apart, 16 columns,
+// emulated: off by 2e-12 of the largest entry without and 1e-16 with it, FP64 sums by 1e-15. The kernel takes 108
+// us with it on the 27-point system, 102 without; 132 with the exponents taken from the diagonal on the way.)
 constexpr int kMxDrainTiles = 7;  // 112 rows between two drains of the FP32 sums into FP64
 
 template <int KP, bool SYM, bool WT = false>
 __global__ void __launch_bounds__(kMxThreads, SYM && KP <= 16 ? 2 : 1)
 k_gram_mx(int n, const double* __restrict__ X, const double* __restrict__ Y, const double* __restrict__ dw,
-          double* __restrict__ part, int pstride, const SolveState* __restrict__ st) {
+          const int* __restrict__ rexp, double* __restrict__ part, int pstride, const SolveState* __restrict__ st) {
   constexpr int KV = 16, WARPS = kMxThreads / 32;
   if (st != nullptr && st->done) return;
   constexpr bool BAL = !SYM;
@@ -550,7 +551,7 @@ k_gram_mx(int n, const double* __restrict__ X, const double* __restrict__ Y, con
   float acc[kMxDigits][2][4];
   double f[2][4];
   int rs[BAL ? 4 : 1];  // r of the tile's rows
-  const int e0 = BAL && dw != nullptr ? mx_exponent(__ldg(dw)) : 0;
+  constexpr int tiny = BAL ? kMxTiny + 64 : kMxTiny;
   int ex[2] = {0, 0}, ey[2] = {0, 0};  // scale exponents of view columns g, g + 8
   auto zero = [&]() {
 #pragma unroll
@@ -576,7 +577,7 @@ k_gram_mx(int n, const double* __restrict__ X, const double* __restrict__ Y, con
         const int el = ex[q >> 1];
         const int ej = __shfl_sync(kMxAll, SYM && KP <= KV ? ex[b] : ey[b], (2 * t + (q & 1)) * 4);
         bool ok;
-        const int k = el + ej - 2044 - 2 * kMxGramBits + 56 - (BAL ? 126 : 0);
+        const int k = el + ej - 2044 - 2 * kMxGramBits + 56;
         double v = ll_to_double_scaled_rn(sum, k, ok);
         if (!ok) v = ldexp(ll_to_double_rn(sum), k);
         f[b][q] += max(el, ej) == kMxNaN ? mx_nan() : v;
@@ -596,7 +597,7 @@ k_gram_mx(int n, const double* __restrict__ X, const double* __restrict__ Y, con
     for (int h = 0; h < 4; ++h) {
       const size_t r = base + 2 * t + (h & 1) + 8 * (h >> 1);
       if constexpr (BAL)
-        rs[h] = dw != nullptr && r < nv ? max(-63, min(63, (mx_exponent(__ldg(dw + r)) - e0) >> 1)) : 0;
+        rs[h] = rexp != nullptr && r < nv ? __ldg(rexp + r) : 0;
 #pragma unroll
       for (int c = 0; c < 2; ++c) {
         const size_t o = r * LD + g + 8 * c;
@@ -607,8 +608,8 @@ k_gram_mx(int n, const double* __restrict__ X, const double* __restrict__ Y, con
       }
     }
   };
-  // X takes part as 2^(63 + r) X and Y as 2^(63 - r) Y
-  auto off = [&](int h, int sign) { return BAL ? 63 + sign * rs[BAL ? h : 0] : 0; };
+  // X takes part as 2^r X and Y as 2^-r Y
+  auto off = [&](int h, int sign) { return BAL ? sign * rs[BAL ? h : 0] : 0; };
   auto grow = [&](const auto& v, int sign, const int (&e)[2], int (&ne)[2]) {
     bool over = false;
 #pragma unroll
@@ -618,7 +619,7 @@ k_gram_mx(int n, const double* __restrict__ X, const double* __restrict__ Y, con
       for (int h = 0; h < 4; ++h) m = max(m, mx_exponent(v[h][c]) + off(h, sign));
       m = max(m, __shfl_xor_sync(kMxAll, m, 1));
       m = max(m, __shfl_xor_sync(kMxAll, m, 2));
-      ne[c] = m > e[c] ? m + 1 : e[c];
+      ne[c] = m > e[c] ? max(m, min(m + 1, 0x7FE)) : e[c];
       over |= ne[c] != e[c];
     }
     return over;
@@ -641,8 +642,8 @@ k_gram_mx(int n, const double* __restrict__ X, const double* __restrict__ Y, con
 #pragma unroll
       for (int c = 0; c < 2; ++c) {
         uint32_t d[kMxDigits];
-        mx_digits(mx_int<kMxGramBits>(v[2 * hh][c], e[c], off(2 * hh, sign)),
-                  mx_int<kMxGramBits>(v[2 * hh + 1][c], e[c], off(2 * hh + 1, sign)), d);
+        mx_digits(mx_int<kMxGramBits>(v[2 * hh][c], e[c], off(2 * hh, sign), tiny),
+                  mx_int<kMxGramBits>(v[2 * hh + 1][c], e[c], off(2 * hh + 1, sign), tiny), d);
 #pragma unroll
         for (int q = 0; q < kMxDigits; ++q) a[q][2 * hh + c] = d[q];
       }

@@ -359,6 +359,15 @@ __global__ void k_check_finite(long long count, const double* __restrict__ v, in
   if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) atomicOr(flag, 4);
 }
 
+// rexp[i] = half the exponent of a_ii relative to a_00, at most 63 either way: 2^rexp is the size of D = diag(sqrt A_jj)
+// for the rows of P and of A P in their Gram (rows_mma.cuh).
+__global__ void k_row_exponents(int n, const double* __restrict__ diag, int* __restrict__ rexp) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const int e0 = (__double2hiint(diag[0]) >> 20) & 0x7FF, e = (__double2hiint(diag[i]) >> 20) & 0x7FF;
+  rexp[i] = max(-63, min(63, (e - e0) >> 1));
+}
+
 // d = 1/sqrt(diag) (= D^{-1} of Section 1), sqd = sqrt(diag) (= D), wdiag = diag (= D^2).
 __global__ void k_make_scaling(int n, const double* __restrict__ diag, double* __restrict__ d,
                                double* __restrict__ sqd) {

@@ -200,3 +200,22 @@ def test_non_finite_initial_block_breaks_down_at_the_set_up(mb, s, value):
     finally:
         sv.close()
     assert (info["status"], info["iterations"]) == (mb.MBPCG_BREAKDOWN, 0)
+
+
+@pytest.mark.parametrize("s,precond", [(4, 0), (8, 0), (16, 0), (11, 1), (32, 0)])
+@pytest.mark.parametrize("power", [-400, 400])
+def test_a_power_of_two_changes_no_bit(mb, s, precond, power):
+    """2^400 A and 2^-400 A: the scales follow, every digit stays. X0 and X~ are 2^-power of those of A, R, W, P and
+    Sigma the same (unscaled; Jacobi scaling takes D = 2^(power / 2) out of X and R besides)."""
+    A = wl.diffusion3d(33, 6) if s > 4 else wl.diffusion3d(41, 6)
+    n = A.n
+    b, U = wl.rhs(n, 0), wl.initial_block(n, s, 1)
+    (one,) = states(mb, A, b, U, s, precond, (2,))
+    B = wl.CSR(n, A.row_ptr, A.col_idx, A.val * 2.0 ** power)
+    (two,) = states(mb, B, b, U, s, precond, (2,))
+    half = 2.0 ** (-power // 2)
+    factor = {"X0": 2.0 ** -power, "Xt": 2.0 ** -power, "R": 1.0, "W": 1.0, "P": 1.0, "Sigma": 1.0}
+    if precond:
+        factor = {"X0": half, "Xt": half, "R": half, "W": 1.0, "P": 1.0, "Sigma": half}
+    for key, f in factor.items():
+        assert np.array_equal(two[key], one[key] * f), key
