@@ -10,7 +10,7 @@
 // side. What binds now is the integer work: about 50 operations per value split or combined. Measured (us per
 // launch, FP64 pipe -> here; the block update with its Gram V^T V):
 //                                    block update        W/P update     Gram P^T (A P) (in the product)
-//   27-point 96^3, KP = 16          1357 -> 234 + 65     408 -> 147      239 -> 108 (102 without balancing)
+//   27-point 96^3, KP = 16          1357 -> 238 + 65     408 -> 147      239 -> 108 (102 without balancing)
 //   diffusion 64^3, KP = 32         1619 -> 299 + 111    471 -> 165      280 -> 125
 //   diffusion 100^3, KP = 8          455 -> 140 + 49     129 -> 85        78 -> 97 (kept fused)
 //   diffusion 128^3, KP = 4          288 -> 152 + 50      77 -> 92 (kept)  58 -> 110 (kept fused)
@@ -529,7 +529,7 @@ k_pw_mx(int n, const double* __restrict__ V, double* __restrict__ W, double* __r
 // the rows would lose what their product does not: the rows are balanced by r = half the exponent of a_ii
 // (rexp, k_row_exponents; or NULL), 2^r X against 2^-r Y. (Two unknowns per point in units 10^6 apart, 16 columns,
 // emulated: off by 2e-12 of the largest entry without and 1e-16 with it, FP64 sums by 1e-15. The kernel takes 108
-// us with it on the 27-point system, 102 without; 132 with the exponents taken from the diagonal on the way.)
+// us with it on the 27-point system, 102 without; 122 to 132 with the exponents taken from the diagonal on the way.)
 constexpr int kMxDrainTiles = 7;  // 112 rows between two drains of the FP32 sums into FP64
 
 template <int KP, bool SYM, bool WT = false>
